@@ -18,7 +18,7 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libsmpq.so")
 OBJ = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE]
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-split-compile=4", "-Xcompiler", "-fPIC", "-I", INCLUDE]
 # extra nvcc flags for tuning sweeps, e.g. SMPQ_NVCC_EXTRA="-DSMPQ_FP32_MIN_BLOCKS=3"
 FLAGS += os.environ.get("SMPQ_NVCC_EXTRA", "").split()
 

@@ -294,9 +294,11 @@ size_t bytes_per_rhs(const smpq_ctx *ctx, int prec, int n_sup, int npoles) {
                                    : (prec == SMPQ_MIXED ? 4 * 16 + 4 * 8 : 3 * 16); // MIXED: p t r x_hi, p t r x_lo
     if (ctx->opt.true_residual && prec == SMPQ_FP64) per += 2 * 16; // x64, t64
     size_t full = (size_t)ctx->V * 12 * per;
-    size_t eb = (prec == SMPQ_FP32 || half) ? 8 : (prec == SMPQ_MIXED ? 16 + 8 : 16); // MIXED: FP64 and FP32 copies
-    size_t sup = (size_t)n_sup * 12 * (npoles * eb + 16);
-    return full + sup;
+    // support: y and the residual history, or as much of that as the fields
+    // take (a shorter history needs the shifted directions beside it)
+    const size_t want = (size_t)n_sup * 12 * hist_bytes_wanted(prec, ctx->opt.max_iter);
+    const size_t dirs = (size_t)n_sup * 12 * npoles * 16;
+    return full + (size_t)n_sup * 12 * 16 + std::min(want, std::max(full, dirs) + dirs);
 }
 
 // kind 0: q^SMP(x) of Eq. 16; kind 1: SMP estimate of diag D_W^{-1}

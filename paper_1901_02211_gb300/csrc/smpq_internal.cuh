@@ -87,7 +87,7 @@ struct smpq_ctx {
 // workspace slots of smpq_ctx::ws
 enum WsId {
     W_P, W_T, W_R, W_XLO, W_XHI, W_T64, W_PS, W_Y, W_PART, W_SCAL, W_B64,
-    W_SRC, W_OUT, W_SUP, W_QTERM, W_RHS, W_Q, W_MISC, W_COUNT
+    W_SRC, W_OUT, W_SUP, W_QTERM, W_RHS, W_Q, W_MISC, W_HIST, W_HCOEF, W_PS32, W_COUNT
 };
 
 // ---------------------------------------------------------------- host helpers
@@ -164,7 +164,26 @@ struct SolveOut {
     double true_resid = -1; // max_j |b - (A + s0) x|/|b| of the base system (-1: not computed)
     float solve_ms = 0;
 };
+// One lattice of a solve, as its caller describes it: the context (geometry,
+// links), the right-hand sides and support (spec), its rational's shifts and
+// where the results go.  A solve of several lattices (the uneven batch) takes
+// precision, tolerance and options from the first lattice's context.
+struct LatIn {
+    smpq_ctx *ctx;
+    const SolveSpec *spec;
+    ShiftParams sp;
+    SolveOut *out;
+};
+
+// one solve in RHS tiles of BC columns (msolve.cuh): tolerance, iteration cap,
+// CG coefficients into hist (Lanczos, nullable), fixed > 0: that many iterations
+template <int BC>
+int solve_bc(const std::vector<LatIn> &lats, double tol, int max_iter, double *hist, int hist_len, int fixed);
+template <int BC> float time_kind_bc(smpq_ctx *ctx, int kind, int B, int tpb, int nr, int reps, void *buf, double *part,
+                                     double *alpha, int *err);
 int multishift_solve(smpq_ctx *ctx, const SolveSpec &spec, SolveOut *out);
+// bytes of residual history per support element that a solve would like
+size_t hist_bytes_wanted(int prec, int max_iter);
 // one solve over n (1..4) lattices of different sizes, their right-hand sides
 // in the same launches (ctxs[0] supplies stream, workspace and options; every
 // spec has the same precision and tile width and its own B, support, sources)
