@@ -203,7 +203,7 @@ Shape tune_shape_raw(smpq_ctx *ctx, int B, int prec, int *cached) {
     const size_t nf = (size_t)B * 12 * ctx->V;
     const bool half = prec == SMPQ_FP16N || prec == SMPQ_BF16N;
     const size_t hb = ((nf * 4 + nf / 12 * 4) + 255) / 256 * 256;
-    const size_t scratch = half ? 2 * hb + nf * sizeof(float2) : 3 * nf * (prec == SMPQ_FP32 ? sizeof(float2) : sizeof(df64c));
+    const size_t scratch = half ? 2 * hb + nf * sizeof(float2) : 3 * nf * (prec == SMPQ_FP32 ? sizeof(float2) : prec == SMPQ_FP64 ? 17 : sizeof(df64c));
     if (ensure(ctx, ctx->ws[W_P], scratch) ||
         ensure(ctx, ctx->ws[W_PART], (size_t)2 * nf / 12 * sizeof(double) + 64) ||
         ensure(ctx, ctx->ws[W_SCAL], (size_t)B * sizeof(double) + 16)) {
@@ -291,7 +291,7 @@ size_t bytes_per_rhs(const smpq_ctx *ctx, int prec, int n_sup, int npoles) {
     const bool half = prec == SMPQ_FP16N || prec == SMPQ_BF16N;
     size_t per = prec == SMPQ_FP32 ? (4 * 8 + 2 * 16)
                  : half            ? (2 * 5 + 2 * 8 + 2 * 16) // p, t: 4 B + a 12th of the 4-byte norm
-                                   : (prec == SMPQ_MIXED ? 4 * 16 + 4 * 8 : 3 * 16); // MIXED: p t r x_hi, p t r x_lo
+                                   : (prec == SMPQ_MIXED ? 4 * 16 + 4 * 8 : 3 * 17); // MIXED: p t r x_hi, p t r x_lo; FP64: p t r, exponents
     if (ctx->opt.true_residual && prec == SMPQ_FP64) per += 2 * 16; // x64, t64
     size_t full = (size_t)ctx->V * 12 * per;
     // support: y and the residual history, or as much of that as the fields
@@ -339,8 +339,13 @@ int compute_classes(smpq_ctx *ctx, const std::vector<int> &classes, double *q_re
         if (kind == 0 && ctx->lm_k > 0) per += (size_t)ctx->V * 12 * sizeof(double2); // projected source field
         long cap = (long)((0.6 * (double)(freeb + held)) / (double)per);
         cap = std::max(12L, cap - cap % 48);
-        B = (int)std::min<long>(nrhs_total, cap);
-        if (B > 48) B -= B % 48;
+        // As few batches as the memory allows, of equal size, in whole 48-column
+        // tiles (972 sources: one batch of 1008; 960 and a second batch of which
+        // 948 columns were padding took twice as long); 24-column ones in FP64,
+        // whose kernels are as fast in them.  Up to 48 sources: as they are.
+        const long nb = (nrhs_total + cap - 1) / cap, tile = prec == SMPQ_FP64 ? 24 : 48;
+        B = (int)std::min<long>(cap, nrhs_total <= 48 ? nrhs_total
+                                                      : ((nrhs_total + nb - 1) / nb + tile - 1) / tile * tile);
     }
     if (B > 1) B -= B % 12;
     if (B < 1) B = 1;
@@ -821,6 +826,7 @@ int smpq_destroy(smpq_ctx *ctx) {
         release(ctx->U64);
         release(ctx->U32);
         release(ctx->Udf);
+        release(ctx->Ubf);
         release(ctx->d_err);
         release(ctx->Uh16);
         release(ctx->Ub16);
@@ -878,6 +884,7 @@ int smpq_load_gauge(smpq_ctx *ctx, const int dims[4], const double *links, int o
     if ((rc = ensure(ctx, ctx->U64, (size_t)V * 36 * sizeof(double2)))) return rc;
     if ((rc = ensure(ctx, ctx->U32, (size_t)V * 36 * sizeof(float2)))) return rc;
     if ((rc = ensure(ctx, ctx->Udf, (size_t)V * 36 * sizeof(df64c)))) return rc;
+    if ((rc = ensure(ctx, ctx->Ubf, (size_t)V * 36 * sizeof(int4)))) return rc;
     if ((rc = ensure(ctx, ctx->Uh16, (size_t)V * 24 * 4))) return rc;
     if ((rc = ensure(ctx, ctx->Ub16, (size_t)V * 24 * 4))) return rc;
     const double *src = links;
@@ -891,7 +898,7 @@ int smpq_load_gauge(smpq_ctx *ctx, const int dims[4], const double *links, int o
     for (int mu = 0; mu < 4; ++mu) ctx->dims[mu] = dims[mu];
     ctx->V = (int)V;
     set_geom(ctx);
-    launch_pack_links(src, (double *)ctx->U64.p, (float *)ctx->U32.p, ctx->Udf.p, (int)V, ctx->stream);
+    launch_pack_links(src, (double *)ctx->U64.p, (float *)ctx->U32.p, ctx->Udf.p, ctx->Ubf.p, (int)V, ctx->stream);
     launch_pack_links12(src, ctx->Uh16.p, ctx->Ub16.p, (int)V, ctx->stream);
     if ((rc = ensure(ctx, ctx->ws[W_PART], 64))) return rc;
     double *derr = (double *)ctx->ws[W_PART].p;
@@ -1077,25 +1084,29 @@ int smpq_dslash(smpq_ctx *ctx, const double *in, double *out, int B, int dagger,
     cudaStream_t st = ctx->stream;
     const size_t n = (size_t)ctx->V * 12 * B;
     const size_t fb = dslash_field_bytes(ctx, precision, B);
-    if ((rc = ensure(ctx, ctx->ws[W_SRC], n * 16 + 2 * fb))) return rc;
-    double *abi = (double *)ctx->ws[W_SRC].p;
-    char *tin = (char *)ctx->ws[W_SRC].p + n * 16, *tout = tin + fb;
+    // host buffers: staged copies of in and out; device: the caller's
+    const size_t bfb = precision == SMPQ_FP64 ? bf_field_bytes(ctx->V, B) : 0;
+    const bool apart = !on_device || in + 2 * n <= out || out + 2 * n <= in;
+    const size_t stage = on_device ? 0 : n * 16;
+    if ((rc = ensure(ctx, ctx->ws[W_SRC], 2 * stage + std::max(2 * fb, bfb)))) return rc;
+    double *abi = (double *)ctx->ws[W_SRC].p + stage / 8;
+    char *tin = (char *)ctx->ws[W_SRC].p + 2 * stage, *tout = tin + fb;
     const double *din = in;
     if (!on_device) {
-        cudaMemcpyAsync(abi, in, n * 16, cudaMemcpyHostToDevice, st);
-        din = abi;
+        cudaMemcpyAsync(ctx->ws[W_SRC].p, in, n * 16, cudaMemcpyHostToDevice, st);
+        din = (const double *)ctx->ws[W_SRC].p;
     }
-    const int BC = 1;
     const void *U = dslash_links(ctx, precision);
     double *dout = on_device ? out : abi;
-    if (precision == SMPQ_FP64) {
-        launch_to_tiled<double>(din, tin, ctx->V, B, BC, st);
-        launch_dslash<double>(ctx->geom, U, tin, tout, B, BC, dagger, ctx->opt.kappa, st);
-        launch_from_tiled<double>(tout, dout, ctx->V, B, BC, st);
+    if (precision == SMPQ_FP64 && apart) {
+        launch_abi_to_bf(din, tin, ctx->V, B, st);
+        launch_dslash_bf(ctx->geom, ctx->Ubf.p, U, tin, din, dout, B, dagger, ctx->opt.kappa, st);
+    } else if (precision == SMPQ_FP64) { // overlapping fields: through copies of both
+        launch_to_tiled<double>(din, tin, ctx->V, B, 1, st);
+        launch_dslash<double>(ctx->geom, U, tin, tout, B, 1, dagger, ctx->opt.kappa, st);
+        launch_from_tiled<double>(tout, dout, ctx->V, B, 1, st);
     } else if (precision == SMPQ_FP32) {
-        launch_to_tiled<float>(din, tin, ctx->V, B, BC, st);
-        launch_dslash<float>(ctx->geom, U, tin, tout, B, BC, dagger, ctx->opt.kappa, st);
-        launch_from_tiled<float>(tout, dout, ctx->V, B, BC, st);
+        launch_dslash_fp32_abi(ctx->geom, U, din, tin, dout, B, dagger, ctx->opt.kappa, st);
     } else {
         launch_to_half(precision, din, tin, ctx->V, B, st);
         launch_dslash_half(precision, ctx->geom, U, tin, tout, B, dagger, ctx->opt.kappa, st);

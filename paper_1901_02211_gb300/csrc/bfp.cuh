@@ -1,0 +1,365 @@
+// D_W in block fixed point: FP64 accuracy on the integer pipe.
+//
+// GB300 executes 2 FP64 operations per clock and SM, but 64 multiply-adds of
+// two 32-bit integers into a 64-bit sum (mad.wide: 2 cycles a warp against 66
+// for an FP64 FMA, measured).  The FP64 iterations therefore keep a site's 24
+// real numbers (12 complex components of one column) as 64-bit integers with
+// one exponent,
+//     value = v * 2^e,  |v| < 2^60, the largest at least 2^59,
+// 7 bits more than a double holds for the largest component (a component that
+// is smaller by 2^k keeps 60 - k bits).  Links are integers in units of 2^-60.
+// A product of two such numbers, each split into a signed high and a signed
+// low word, is three mad.wide into 64-bit sums (high; middle twice); low times
+// low, about 2^-57 of the largest, is left out.  Sums are exact, so the hop's
+// error is that of its truncations, about 2^-56 of the largest component of
+// the nine sites, against 2^-53 of every partial sum in FP64.
+//   Bounds: a projected component is below 2^61, so its words are below 2^29
+// and 2^31, a link's 2^28 and 2^31.  Six products in a middle sum stay below
+// 6 * 2^60 + sqrt(6) * 2^59 < 2^63; the rows of a link have norm 1, so a hop's
+// high sum, in units of 2^64, is below sqrt(6) * 2^(61 + 60 - 64) and eight
+// hops below 2^61.3.
+//
+// Cycles a warp for one site and 32 columns: 8 hops of 228 mad.wide (2), 36
+// shifts and splits (4 and 3), 36 64-bit additions (2) and 21 loads come to
+// 5500; the 960 FP64 instructions that they replace take 63 000.
+#pragma once
+#include "wilson.cuh"
+
+struct __align__(16) bfc {
+    long long x, y;
+};
+// a field of n complex values: the components, then one exponent per site and column
+struct BFF {
+    bfc *v;
+    int *e;
+};
+constexpr int BF_ZERO = -(1 << 28); // exponent of a site whose components are all 0
+constexpr int BF_BAD = 1 << 28;     // of one that holds an infinity or a NaN
+
+struct bf {}; // names the format where a template takes an iteration type
+
+// component c of site s in an RHS tile: [site][12][BC], or [12][site] for
+// one-column tiles (neighbouring threads then read neighbouring sites)
+template <int BC> struct BfOff {
+    int V;
+    __device__ __forceinline__ size_t operator()(int s, int c) const {
+        if constexpr (BC == 1) return (size_t)c * V + s;
+        else return ((size_t)s * 12 + c) * BC;
+    }
+    __device__ __forceinline__ size_t exp(int s) const { return (size_t)s * BC; }
+};
+// the caller's layout [site][12][B] with B only known at run time
+template <> struct BfOff<0> {
+    int V, B;
+    __device__ __forceinline__ size_t operator()(int s, int c) const { return ((size_t)s * 12 + c) * B; }
+    __device__ __forceinline__ size_t exp(int s) const { return (size_t)s * B; }
+};
+
+// c + a * b in one instruction (the compiler would turn a factor -a into a
+// product and a 64-bit subtraction)
+__device__ __forceinline__ long long madw(int a, int b, long long c) {
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+// 1 that the compiler does not know: high + one * middle is then one mad.wide
+// instead of a sign extension and a 64-bit addition
+__device__ __forceinline__ int opaque_one() {
+    int v;
+    asm("mov.u32 %0, 1;" : "=r"(v));
+    return v;
+}
+// x = h * 2^32 + l with both signed
+__device__ __forceinline__ void bf_split(long long x, int &h, int &l) {
+    l = (int)x;
+    h = (int)(x >> 32) + (int)((unsigned)l >> 31);
+}
+constexpr long long BF_HALF = 0x80000000ll; // rounds the middle sum
+
+// a real factor m * 2^e, 2^61 <= |m| < 2^62 (or 0)
+struct BfScal {
+    int h, l, e;
+};
+__host__ __device__ __forceinline__ BfScal bf_scal(double s) {
+    unsigned long long u;
+#ifdef __CUDA_ARCH__
+    u = (unsigned long long)__double_as_longlong(s);
+#else
+    __builtin_memcpy(&u, &s, 8);
+#endif
+    const int eb = (int)(u >> 52) & 0x7ff;
+    long long m = eb ? (long long)((u & 0xfffffffffffffull) | 0x10000000000000ull) << 9 : 0;
+    if (u >> 63) m = -m;
+    BfScal r;
+    r.l = (int)m;
+    r.h = (int)(m >> 32) + (int)((unsigned)r.l >> 31);
+    r.e = eb - 1075 - 9;
+    if (eb == 0x7ff) r.e = BF_BAD; // infinity or NaN: the result is marked bad
+    return r;
+}
+// x * s / 2^64 (the exponents add up to e_x + s.e + 64); |result| < |x| / 4
+__device__ __forceinline__ long long bf_mul(long long x, const BfScal &s, int one) {
+    int h, l;
+    bf_split(x, h, l);
+    const long long mid = madw(h, s.l, madw(l, s.h, BF_HALF));
+    return madw((int)(mid >> 32), one, madw(h, s.h, 0));
+}
+// arithmetic right shift by any n >= 0
+__device__ __forceinline__ long long bf_shr(long long x, int n) { return x >> min(n, 63); }
+
+// v * 2^e as a double
+__device__ __forceinline__ double bf_double(long long v, int e) {
+    const double d = __ll2double_rn(v);
+    const int hi = __double2hiint(d), eb = ((hi >> 20) & 0x7ff) + e;
+    if (v == 0) return 0.0;
+    if (eb < 1 || eb > 2046) return e >= BF_BAD / 2 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(d, e);
+    return __hiloint2double(hi + (e << 20), __double2loint(d));
+}
+
+// 24 doubles as a block (e = BF_BAD if some are not finite); wide: the nonzero
+// ones span more than 2^40
+__device__ __forceinline__ void bf_from_double(const double2 d[12], bfc v[12], int &e, bool &wide) {
+    int top = 0, low = 0x7ff;
+    bool any = false;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const double q[2] = {d[c].x, d[c].y};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int eb = max((__double2hiint(q[k]) >> 20) & 0x7ff, 1);
+            if (q[k] != 0) {
+                any = true;
+                low = min(low, eb);
+            }
+            top = max(top, eb);
+        }
+    }
+    wide = any && top - low > 40;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const double q[2] = {d[c].x, d[c].y};
+        long long r[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const long long u = __double_as_longlong(q[k]);
+            const int eb = (int)(u >> 52) & 0x7ff;
+            const long long m = ((u & 0xfffffffffffffll) | (eb ? 0x10000000000000ll : 0)) << 7;
+            const long long a = bf_shr(m, top - max(eb, 1));
+            r[k] = u < 0 ? -a : a;
+        }
+        v[c] = bfc{r[0], r[1]};
+    }
+    e = top == 0x7ff ? BF_BAD : any ? top - 1082 : BF_ZERO;
+}
+
+// Brings a block with |v| < 2^60 and exponent e to the normal form.
+__device__ __forceinline__ void bf_normalise(bfc v[12], int &e) {
+    int mx = 0, mn = -1;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const int a = (int)(v[c].x >> 32), b = (int)(v[c].y >> 32);
+        mx = max(mx, max(a, b));
+        mn = min(mn, min(a, b));
+    }
+    const int m = max(mx, ~mn);
+    if (m == 0) { // all below 2^32: is there anything?
+        int any = 0;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) any |= (int)v[c].x | (int)v[c].y;
+        if (any == 0 && e < BF_BAD / 2) e = BF_ZERO;
+    }
+    const int sh = max(__clz(m) - 4, 0);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) v[c] = bfc{v[c].x << sh, v[c].y << sh};
+    if (e > BF_ZERO / 2) e -= sh;
+    if (e >= BF_BAD / 2) e = BF_BAD;
+}
+
+// sum of the squares of a block in normal form
+__device__ __forceinline__ double bf_norm2(const bfc v[12], int e, int one) {
+    if (e <= BF_ZERO / 2) return 0.0;
+    if (e >= BF_BAD / 2) return __longlong_as_double(0x7ff8000000000000ll);
+    long long hi = 0, lo = 0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) { // twelve products of 2^59 fit the middle sum
+        long long mid = BF_HALF;
+#pragma unroll
+        for (int c = 6 * g; c < 6 * g + 6; ++c) {
+            int h, l;
+            bf_split(v[c].x, h, l);
+            hi = madw(h, h, hi);
+            mid = madw(h, l, mid);
+            bf_split(v[c].y, h, l);
+            hi = madw(h, h, hi);
+            mid = madw(h, l, mid);
+        }
+        lo = madw((int)(mid >> 32), one, lo);
+    }
+    return bf_double(hi + 2 * lo, 64 + 2 * e);
+}
+
+// ---------------------------------------------------------------- the hop
+// h = (psi_0 + G S_mu psi_lo, ...) of one colour (p0..p3: its four spin components)
+template <int MU, int G> __device__ __forceinline__ void bf_project(bfc p0, bfc p1, bfc p2, bfc p3, bfc &h0, bfc &h1) {
+    bfc s0, s1;
+    if (MU == 0) { s0 = {p3.y, -p3.x}; s1 = {p2.y, -p2.x}; }
+    else if (MU == 1) { s0 = {-p3.x, -p3.y}; s1 = {p2.x, p2.y}; }
+    else if (MU == 2) { s0 = {p2.y, -p2.x}; s1 = {-p3.y, p3.x}; }
+    else { s0 = p2; s1 = p3; }
+    h0 = {p0.x + G * s0.x, p0.y + G * s0.y};
+    h1 = {p1.x + G * s1.x, p1.y + G * s1.y};
+}
+// lower half += G S_mu^dag w
+template <int MU, int G> __device__ __forceinline__ void bf_lower(bfc w0, bfc w1, bfc &l0, bfc &l1) {
+    bfc a, b;
+    if (MU == 0) { a = {-w1.y, w1.x}; b = {-w0.y, w0.x}; }
+    else if (MU == 1) { a = w1; b = {-w0.x, -w0.y}; }
+    else if (MU == 2) { a = {-w0.y, w0.x}; b = {w1.y, -w1.x}; }
+    else { a = w0; b = w1; }
+    l0 = {l0.x + G * a.x, l0.y + G * a.y};
+    l1 = {l1.x + G * b.x, l1.y + G * b.y};
+}
+
+// acc += (1 + G g_mu) U psi(nb) (back = false, G = DAG ? 1 : -1) or (1 - G g_mu)
+// U^dag psi(nb) (back = true; as the conjugate of U^T conj(h)), its sign flipped
+// if flip; psi's block is shifted right by n bits to the common exponent, acc in
+// units of 2^4 of that.  The orientation is a run-time value: one copy of this
+// code for each direction fits the instruction cache, eight do not (measured:
+// 210 against 178 ms for six classes of 8^3x16, "no instruction" the first stall).
+// links: int4 {re high, re low, im high, im low} per element
+template <int MU, bool DAG, typename Off>
+__device__ __forceinline__ void bf_hop(bool back, const int4 *__restrict__ U, const bfc *__restrict__ in,
+                                          const Off &off, int Vl, int nb, int ls, int n, bool flip, int one,
+                                          bfc acc[12]) {
+    constexpr int GF = DAG ? 1 : -1;
+    int hh[2][3][2], hl[2][3][2];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const bfc p0 = in[off(nb, a)], p1 = in[off(nb, 3 + a)], p2 = in[off(nb, 6 + a)], p3 = in[off(nb, 9 + a)];
+        bfc h0, h1;
+        if (back) {
+            bf_project<MU, -GF>(p0, p1, p2, p3, h0, h1);
+            h0.y = -h0.y;
+            h1.y = -h1.y;
+        } else {
+            bf_project<MU, GF>(p0, p1, p2, p3, h0, h1);
+        }
+        if (flip) {
+            h0 = {-h0.x, -h0.y};
+            h1 = {-h1.x, -h1.y};
+        }
+        bf_split(h0.x >> n, hh[0][a][0], hl[0][a][0]);
+        bf_split(h0.y >> n, hh[0][a][1], hl[0][a][1]);
+        bf_split(h1.x >> n, hh[1][a][0], hl[1][a][0]);
+        bf_split(h1.y >> n, hh[1][a][1], hl[1][a][1]);
+    }
+    const int4 *ul = U + ((size_t)MU * Vl + ls) * 9;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        int4 u[3];
+        if (back) {
+#pragma unroll
+            for (int b = 0; b < 3; ++b) u[b] = ul[b * 3 + a];
+        } else {
+#pragma unroll
+            for (int b = 0; b < 3; ++b) u[b] = ul[a * 3 + b];
+        }
+        bfc w[2];
+        long long rh[2] = {0, 0}, rm[2] = {BF_HALF, BF_HALF}, ih[2] = {0, 0}, im[2] = {BF_HALF, BF_HALF};
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int ah = -u[b].z, al = -u[b].w;
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                rh[s] = madw(u[b].x, hh[s][b][0], madw(ah, hh[s][b][1], rh[s]));
+                rm[s] = madw(u[b].x, hl[s][b][0], madw(u[b].y, hh[s][b][0], rm[s]));
+                rm[s] = madw(ah, hl[s][b][1], madw(al, hh[s][b][1], rm[s]));
+                ih[s] = madw(u[b].x, hh[s][b][1], madw(u[b].z, hh[s][b][0], ih[s]));
+                im[s] = madw(u[b].x, hl[s][b][1], madw(u[b].y, hh[s][b][1], im[s]));
+                im[s] = madw(u[b].z, hl[s][b][0], madw(u[b].w, hh[s][b][0], im[s]));
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+            w[s] = {madw((int)(rm[s] >> 32), one, rh[s]), madw((int)(im[s] >> 32), one, ih[s])};
+        if (back) {
+            acc[a] = {acc[a].x + w[0].x, acc[a].y - w[0].y};
+            acc[3 + a] = {acc[3 + a].x + w[1].x, acc[3 + a].y - w[1].y};
+            bf_lower<MU, -GF>(bfc{w[0].x, -w[0].y}, bfc{w[1].x, -w[1].y}, acc[6 + a], acc[9 + a]);
+        } else {
+            acc[a] = {acc[a].x + w[0].x, acc[a].y + w[0].y};
+            acc[3 + a] = {acc[3 + a].x + w[1].x, acc[3 + a].y + w[1].y};
+            bf_lower<MU, GF>(w[0], w[1], acc[6 + a], acc[9 + a]);
+        }
+    }
+}
+
+// acc * 2^(eref + 4) = hop(s); eref = the largest exponent of s and its neighbours
+template <bool DAG, typename Off>
+__device__ __forceinline__ void bf_wilson(const Geom &g, const int4 *__restrict__ U, const bfc *__restrict__ in,
+                                          const int *__restrict__ ein, const Off &off, int s, int one, bfc acc[12],
+                                          int &eown, int &eref) {
+    const SiteCoords xc(g, s);
+    int nbk[8];
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        const int n = g.n[mu], st = g.stride[mu], c = xc.x[mu];
+        nbk[2 * mu] = c == n - 1 ? s - (n - 1) * st : s + st;
+        nbk[2 * mu + 1] = c == 0 ? s + (n - 1) * st : s - st;
+    }
+    int en[8];
+    eown = eref = ein[off.exp(s)];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        en[k] = ein[off.exp(nbk[k])];
+        eref = max(eref, en[k]);
+    }
+#pragma unroll
+    for (int c = 0; c < 12; ++c) acc[c] = {0, 0};
+    auto dir = [&](auto mc) {
+        constexpr int MU = decltype(mc)::value;
+        const int n = g.n[MU], c = xc.x[MU];
+        const bool anti = g.bcf[MU] < 0;
+        // forward: (1 - g) [DAG: (1 + g)], backward: (1 + g) [DAG: (1 - g)]
+#pragma unroll 1
+        for (int bk = 0; bk < 2; ++bk) {
+            const bool back = bk != 0;
+            const int nb = back ? nbk[2 * MU + 1] : nbk[2 * MU];
+            const int en1 = back ? en[2 * MU + 1] : en[2 * MU];
+            bf_hop<MU, DAG>(back, U, in, off, g.V, nb, back ? nb : s, min(eref - en1, 63),
+                               anti && c == (back ? 0 : n - 1), one, acc);
+        }
+    };
+    dir(std::integral_constant<int, 0>());
+    dir(std::integral_constant<int, 1>());
+    dir(std::integral_constant<int, 2>());
+    dir(std::integral_constant<int, 3>());
+}
+
+// x = own - kappa acc in units of 2^eu, eu at least `least` (>= eown + 2, the
+// exponent of the block own); |x| < 2^60
+__device__ __forceinline__ void bf_dw(const bfc own[12], int eown, const bfc acc[12], int eref, const BfScal &k,
+                                      int least, int one, bfc x[12], int &eu) {
+    const int eq = eref <= BF_ZERO / 2 ? BF_ZERO : eref + 4 + k.e + 64;
+    eu = max(eq, least);
+    const int n = eu - eown, m = eu - eq;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        long long qx = bf_mul(acc[c].x, k, one), qy = bf_mul(acc[c].y, k, one);
+        if (m) { // (only for a tiny kappa)
+            qx = bf_shr(qx, m);
+            qy = bf_shr(qy, m);
+        }
+        x[c] = {bf_shr(own[c].x, n) - qx, bf_shr(own[c].y, n) - qy};
+    }
+    if (eref >= BF_BAD / 2) eu = BF_BAD;
+}
+
+// thread -> (site, column) of the block-fixed-point kernels: blocks of about a
+// hundred threads, so that small lattices reach every SM (24 576 sites and
+// columns are 384 blocks); 128 registers a thread
+template <int BC> struct BfMap {
+    static constexpr int SPB = BC == 1 ? 64 : BC == 12 ? 8 : BC == 24 ? 4 : 5;
+    static constexpr int THREADS = BC * SPB;
+    static constexpr int BLOCKS = 512 / THREADS; // per SM
+};

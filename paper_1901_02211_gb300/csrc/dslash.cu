@@ -2,6 +2,7 @@
 // dslash D_W / D_W^dag (Sec. 2.1, around Eq. 3) used by smpq_dslash.
 #include <string>
 
+#include "bfp.cuh"
 #include "smpq_internal.cuh"
 #include "stage.cuh"
 #include "wilson.cuh"
@@ -9,7 +10,7 @@
 // ------------------------------------------------------------------ links
 // U_aos: double[V][4][3][3][2] -> U64/U32: [(mu * V + s) * 9 + e] complex
 __global__ void pack_links_kernel(const double2 *__restrict__ Uaos, double2 *__restrict__ U64,
-                                  float2 *__restrict__ U32, df64c *__restrict__ Udf, int V) {
+                                  float2 *__restrict__ U32, df64c *__restrict__ Udf, int4 *__restrict__ Ubf, int V) {
     long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (i >= (long)V * 36) return;
     int s = (int)(i / 36), k = (int)(i % 36); // k = mu*9 + e
@@ -18,12 +19,21 @@ __global__ void pack_links_kernel(const double2 *__restrict__ Uaos, double2 *__r
     U64[o] = u;
     U32[o] = make_float2((float)u.x, (float)u.y);
     Udf[o] = df64c{df64(u.x), df64(u.y)};
+    // units of 2^-60 as two signed words; the low one can be negated
+    const double q[2] = {u.x, u.y};
+    int w[4];
+    for (int k = 0; k < 2; ++k) {
+        const double c = fmin(fmax(q[k], -2.0), 2.0); // (a link that is not SU(3) is refused afterwards)
+        bf_split(__double2ll_rn(c * 1152921504606846976.0), w[2 * k], w[2 * k + 1]);
+        if (w[2 * k + 1] == (int)0x80000000) w[2 * k + 1] += 1;
+    }
+    Ubf[o] = make_int4(w[0], w[1], w[2], w[3]);
 }
 
-void launch_pack_links(const double *U_aos, double *U64, float *U32, void *Udf, int V, cudaStream_t st) {
+void launch_pack_links(const double *U_aos, double *U64, float *U32, void *Udf, void *Ubf, int V, cudaStream_t st) {
     long n = (long)V * 36;
     pack_links_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const double2 *)U_aos, (double2 *)U64,
-                                                                     (float2 *)U32, (df64c *)Udf, V);
+                                                                     (float2 *)U32, (df64c *)Udf, (int4 *)Ubf, V);
 }
 
 // max over links of max(|U U^dag - 1|, |det U - 1|), as the bit pattern of a
@@ -233,6 +243,139 @@ template void launch_dslash<double>(const Geom &, const void *, const void *, vo
 template void launch_dslash<float>(const Geom &, const void *, const void *, void *, int, int, int, double,
                                    cudaStream_t);
 
+// ------------------------------------------------------------------ D_W on the caller's fields
+// The ABI layout [V][12][B] is one RHS tile of B columns, so the stencil reads it
+// as it is: the input is converted once (to block fixed point, bfp.cuh, or to
+// FP32), and the stencil writes the caller's doubles.  Before, the fields went
+// through one-column tiles: 209 us of FP64 instructions for 12 columns of 8^3x16
+// between two transposes, 70 us for one column of 4^4 (a single block).
+__global__ void __launch_bounds__(128) abi_to_bf_kernel(const double2 *__restrict__ in, bfc *__restrict__ v,
+                                                        int *__restrict__ e, int V, int B) {
+    const long i = blockIdx.x * 128l + threadIdx.x;
+    if (i >= (long)V * B) return;
+    const int s = (int)(i / B), j = (int)(i % B);
+    const size_t base = (size_t)s * 12 * B + j;
+    double2 d[12];
+    bfc b[12];
+    int x;
+    bool wide;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) d[c] = in[base + (size_t)c * B];
+    bf_from_double(d, b, x, wide);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) v[base + (size_t)c * B] = b[c];
+    // not finite, or components more than 2^40 apart: the sites that read it are done in FP64
+    e[i] = wide ? BF_BAD : x;
+}
+
+// D_W at one site and column in FP64 (what block fixed point does not hold)
+static __device__ __noinline__ void dw_site_fp64(const Geom &g, const double2 *__restrict__ U,
+                                                 const double2 *__restrict__ in, double2 *__restrict__ out, int s,
+                                                 int B, int dagger, double kappa) {
+    double2 acc[12][1];
+    if (dagger) wilson_hop<double, true, 0>(g, U, in, s, acc, B);
+    else wilson_hop<double, false, 0>(g, U, in, s, acc, B);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const size_t o = ((size_t)s * 12 + c) * B;
+        double2 v = in[o];
+        v.x -= kappa * acc[c][0].x;
+        v.y -= kappa * acc[c][0].y;
+        out[o] = v;
+    }
+}
+
+// one thread per site and column in blocks of 32 (few columns: every warp on an
+// SM of its own) or 128 threads; bound by the integer pipe
+template <bool DAG>
+__global__ void __launch_bounds__(128, 4)
+    dslash_bf_kernel(Geom g, const int4 *__restrict__ Ubf, const double2 *__restrict__ U64, const bfc *__restrict__ v,
+                     const int *__restrict__ e, const double2 *__restrict__ in, double2 *__restrict__ out, int B,
+                     BfScal ks, double kappa) {
+    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (i >= (long)g.V * B) return;
+    const int s = (int)(i / B), j = (int)(i % B);
+    const BfOff<0> off{g.V, B};
+    const int one = opaque_one();
+    bfc acc[12], own[12];
+    int eown, eref, eu;
+    bf_wilson<DAG>(g, Ubf, v + j, e + j, off, s, one, acc, eown, eref);
+    if (eref >= BF_BAD / 2) {
+        dw_site_fp64(g, U64, in + j, out + j, s, B, DAG, kappa);
+        return;
+    }
+#pragma unroll
+    for (int c = 0; c < 12; ++c) own[c] = v[j + off(s, c)];
+    bf_dw(own, eown, acc, eref, ks, eown + 2, one, acc, eu);
+#pragma unroll
+    for (int c = 0; c < 12; ++c)
+        out[j + off(s, c)] = make_double2(bf_double(acc[c].x, eu), bf_double(acc[c].y, eu));
+}
+
+size_t bf_field_bytes(int V, int B) { return (size_t)V * B * (12 * sizeof(bfc) + sizeof(int)); }
+
+void launch_abi_to_bf(const double *in, void *field, int V, int B, cudaStream_t st) {
+    const long n = (long)V * B;
+    bfc *v = (bfc *)field;
+    abi_to_bf_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>((const double2 *)in, v, (int *)(v + 12 * n), V, B);
+}
+void launch_dslash_bf(const Geom &g, const void *Ubf, const void *U64, const void *field, const double *in,
+                      double *out, int B, int dagger, double kappa, cudaStream_t st) {
+    const long n = (long)g.V * B;
+    const int th = n < 152 * 128 * 4 ? 32 : 128;
+    const unsigned nb = (unsigned)((n + th - 1) / th);
+    const bfc *v = (const bfc *)field;
+    const int *e = (const int *)(v + 12 * n);
+    const BfScal ks = bf_scal(kappa);
+    if (dagger)
+        dslash_bf_kernel<true><<<nb, th, 0, st>>>(g, (const int4 *)Ubf, (const double2 *)U64, v, e,
+                                                  (const double2 *)in, (double2 *)out, B, ks, kappa);
+    else
+        dslash_bf_kernel<false><<<nb, th, 0, st>>>(g, (const int4 *)Ubf, (const double2 *)U64, v, e,
+                                                   (const double2 *)in, (double2 *)out, B, ks, kappa);
+}
+
+__global__ void __launch_bounds__(256) abi_to_float_kernel(const double2 *__restrict__ in, float2 *__restrict__ out,
+                                                           size_t n) {
+    const size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
+    if (i < n) {
+        const double2 v = in[i];
+        out[i] = make_float2((float)v.x, (float)v.y);
+    }
+}
+template <bool DAG>
+__global__ void __launch_bounds__(128, 6)
+    dslash_abi_kernel(Geom g, const float2 *__restrict__ U, const float2 *__restrict__ in, double2 *__restrict__ out,
+                      int B, float kappa) {
+    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (i >= (long)g.V * B) return;
+    const int s = (int)(i / B), j = (int)(i % B);
+    float2 acc[12][1];
+    wilson_hop<float, DAG, 0>(g, U, in + j, s, acc, B);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const size_t o = ((size_t)s * 12 + c) * B + j;
+        float2 v = in[o];
+        v.x -= kappa * acc[c][0].x;
+        v.y -= kappa * acc[c][0].y;
+        out[o] = make_double2(exact_d(v.x), exact_d(v.y));
+    }
+}
+void launch_dslash_fp32_abi(const Geom &g, const void *U, const double *in, void *field, double *out, int B,
+                            int dagger, double kappa, cudaStream_t st) {
+    const long n = (long)g.V * B;
+    abi_to_float_kernel<<<(unsigned)((12 * n + 255) / 256), 256, 0, st>>>((const double2 *)in, (float2 *)field,
+                                                                          (size_t)12 * n);
+    const int th = n < 152 * 128 * 4 ? 32 : 128;
+    const unsigned nb = (unsigned)((n + th - 1) / th);
+    if (dagger)
+        dslash_abi_kernel<true><<<nb, th, 0, st>>>(g, (const float2 *)U, (const float2 *)field, (double2 *)out, B,
+                                                   (float)kappa);
+    else
+        dslash_abi_kernel<false><<<nb, th, 0, st>>>(g, (const float2 *)U, (const float2 *)field, (double2 *)out, B,
+                                                    (float)kappa);
+}
+
 // ------------------------------------------------------------------ allocation-free dslash
 // smpq_dslash_noalloc keeps its scratch (the tiled copies of the input and the
 // output field that the kernel reads and writes) in this file-scope device
@@ -297,14 +440,17 @@ extern "C" int smpq_dslash_noalloc(smpq_ctx *ctx, const double *in, double *out,
         }
         char *tin = (char *)scratch, *tout = (char *)scratch + half;
         const int BC = 1;
-        if (precision == SMPQ_FP64) {
+        const bool apart = in + 2 * n <= out || out + 2 * n <= in;
+        // (a block-fixed-point field is a 48th larger than the FP64 one: it fits where two of those do)
+        if (precision == SMPQ_FP64 && apart) {
+            launch_abi_to_bf(in, scratch, ctx->V, B, st);
+            launch_dslash_bf(ctx->geom, ctx->Ubf.p, ctx->U64.p, scratch, in, out, B, dagger, ctx->opt.kappa, st);
+        } else if (precision == SMPQ_FP32) { // (the input is copied before anything is written)
+            launch_dslash_fp32_abi(ctx->geom, ctx->U32.p, in, scratch, out, B, dagger, ctx->opt.kappa, st);
+        } else {
             launch_to_tiled<double>(in, tin, ctx->V, B, BC, st);
             launch_dslash<double>(ctx->geom, ctx->U64.p, tin, tout, B, BC, dagger, ctx->opt.kappa, st);
             launch_from_tiled<double>(tout, out, ctx->V, B, BC, st);
-        } else {
-            launch_to_tiled<float>(in, tin, ctx->V, B, BC, st);
-            launch_dslash<float>(ctx->geom, ctx->U32.p, tin, tout, B, BC, dagger, ctx->opt.kappa, st);
-            launch_from_tiled<float>(tout, out, ctx->V, B, BC, st);
         }
         cudaError_t e = cudaStreamSynchronize(st);
         rc = e != cudaSuccess ? cuda_check(ctx, e, "dslash_noalloc") : cuda_check(ctx, cudaGetLastError(), "dslash_noalloc launch");

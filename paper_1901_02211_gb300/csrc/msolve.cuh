@@ -34,6 +34,7 @@
 #include <cmath>
 #include <cstdio>
 
+#include "bfp.cuh"
 #include "half.cuh"
 #include "smpq_internal.cuh"
 #include "stage.cuh"
@@ -62,15 +63,14 @@ template <> struct MinBlocks<df64> { static constexpr int value = SMPQ_DF64_MIN_
 
 // link copy matching the iteration precision
 template <typename T> struct Links;
-template <> struct Links<double> { static const void *get(const smpq_ctx *c) { return c->U64.p; } };
+template <> struct Links<double> { static const void *get(const smpq_ctx *c) { return c->Ubf.p; } }; // (block fixed point)
 template <> struct Links<float> { static const void *get(const smpq_ctx *c) { return c->U32.p; } };
 template <> struct Links<df64> { static const void *get(const smpq_ctx *c) { return c->Udf.p; } };
 
 
 // ------------------------------------------------------------------ block reduction per column
-template <int BC>
+template <int BC, int THREADS = TileMap<BC>::THREADS>
 __device__ __forceinline__ double block_sum(double v, double *sm) {
-    constexpr int THREADS = TileMap<BC>::THREADS;
     double s = 0;
     if constexpr (32 % BC == 0) {
 #pragma unroll
@@ -157,103 +157,133 @@ template <bool M> __device__ __forceinline__ int lat_index(const Lats &L) {
     return l;
 }
 
-// ------------------------------------------------------------------ scalar steps (one thread per column)
-// First scalar step of column j: alpha and the shift recurrences zeta_{k+1},
-// alpha_i (tt = |D_W p|^2, pp = |p|^2, so <p, A p> = tt + s0 pp).
-__device__ void s1_column(int j, double tt, double pp, const Scal &sc, const ShiftParams &sp, int B) {
-    if (j == 0) {
-        sc.flags[0] = 0;
-        sc.flags[3] = 0;
-        if (sc.hist) {
-            int it = sc.iter_counter[0];
-            if (it < sc.hist_len) sc.hist[it] = 0; // filled below when rhs 0 is active
+// ------------------------------------------------------------------ scalar steps
+// Run by one block of NT threads for the BC columns of an RHS tile (from the
+// solve's column j0): thread t < BC has column t's sum and does the column's
+// own scalars, then NT / BC threads share its shifts (one thread per column took 14
+// of them in a row, divisions and dependent loads: 5 us at the end of every
+// D_W launch).
+// First step: alpha and the shift recurrences zeta_{k+1}, alpha_i (tt = |D_W
+// p|^2, pp = |p|^2, so <p, A p> = tt + s0 pp).
+template <int BC, int NT>
+__device__ void s1_tile(int j0, double tt, double pp, const Scal &sc, const ShiftParams &sp, int B, double *sm) {
+    __shared__ int mode[BC]; // 0 idle, 1 active
+    const int t = threadIdx.x;
+    if (t < BC) {
+        const int j = j0 + t;
+        if (j == 0) {
+            sc.flags[0] = 0;
+            sc.flags[3] = 0;
+            if (sc.hist) {
+                int it = sc.iter_counter[0];
+                if (it < sc.hist_len) sc.hist[it] = 0; // filled below when rhs 0 is active
+            }
         }
+        int m = sc.act_rhs[j] != 0;
+        double a = 0;
+        if (m) {
+            const double pAp = tt + sp.s0 * pp;
+            if (!(pAp > 0) || !isfinite(pAp)) {
+                atomicOr(&sc.flags[2], 1);
+                sc.act_rhs[j] = 0;
+                m = 0;
+            } else {
+                a = sc.rr[j] / pAp;
+                if (sc.hist && j == 0) {
+                    int it = sc.iter_counter[0];
+                    if (it < sc.hist_len) sc.hist[it] = a;
+                }
+            }
+        }
+        sc.alpha[j] = a;
+        sc.upd_rhs[j] = m;
+        mode[t] = m;
+        sm[t] = a;
     }
-    const size_t row = (size_t)sc.slot[j] * sp.n * B + j;
-    if (!sc.act_rhs[j]) {
-        sc.alpha[j] = 0;
-        sc.upd_rhs[j] = 0;
-        for (int i = 0; i < sp.n; ++i) { sc.upd[i * B + j] = 0; sc.ha[row + (size_t)i * B] = 0; }
-        return;
-    }
-    double pAp = tt + sp.s0 * pp;
-    if (!(pAp > 0) || !isfinite(pAp)) {
-        atomicOr(&sc.flags[2], 1);
-        sc.alpha[j] = 0;
-        sc.upd_rhs[j] = 0;
-        sc.act_rhs[j] = 0;
-        for (int i = 0; i < sp.n; ++i) { sc.upd[i * B + j] = 0; sc.ha[row + (size_t)i * B] = 0; }
-        return;
-    }
-    double a = sc.rr[j] / pAp;
-    sc.alpha[j] = a;
-    sc.upd_rhs[j] = 1;
-    if (sc.hist && j == 0) {
-        int it = sc.iter_counter[0];
-        if (it < sc.hist_len) sc.hist[it] = a;
-    }
-    double ap = sc.alpha_prev[j], bp = sc.beta_prev[j];
-    for (int i = 0; i < sp.n; ++i) {
-        int ix = i * B + j;
-        const size_t hx = row + (size_t)i * B;
-        if (!sc.act[ix]) { sc.upd[ix] = 0; sc.ha[hx] = 0; continue; }
-        double z = sc.zeta[ix], zp = sc.zeta_prev[ix];
-        double den = a * bp * (zp - z) + zp * ap * (1.0 + sp.sig[i] * a);
-        double zn = z * zp * ap / den;
-        sc.hz[hx] = zn;
-        sc.ha[hx] = a * zn / z;
-        sc.upd[ix] = 1;
+    __syncthreads();
+    constexpr int K = NT / BC;
+    const int q = t % BC, j = j0 + q;
+    if (t < K * BC) {
+        const size_t row = (size_t)sc.slot[j] * sp.n * B + j;
+        const bool on = mode[q];
+        const double a = sm[q], ap = sc.alpha_prev[j], bp = sc.beta_prev[j];
+        for (int i = t / BC; i < sp.n; i += K) {
+            const int ix = i * B + j;
+            const size_t hx = row + (size_t)i * B;
+            if (!on || !sc.act[ix]) { sc.upd[ix] = 0; sc.ha[hx] = 0; continue; }
+            double z = sc.zeta[ix], zp = sc.zeta_prev[ix];
+            double den = a * bp * (zp - z) + zp * ap * (1.0 + sp.sig[i] * a);
+            double zn = z * zp * ap / den;
+            sc.hz[hx] = zn;
+            sc.ha[hx] = a * zn / z;
+            sc.upd[ix] = 1;
+        }
     }
 }
 
-// Second scalar step of column j (rrn = |r_{k+1}|^2): beta, beta_i, the
-// convergence of every shift, the residual-replacement request and the count
-// of columns still above the precision-switch residual.
-__device__ void s2_column(int j, double rrn, const Scal &sc, const ShiftParams &sp, int B, double tol2,
-                          double delta2, double theta2) {
-    if (j == 0) {
-        if (sc.hist) {
-            int it = sc.iter_counter[0];
-            if (it < sc.hist_len) sc.hist[sc.hist_len + it] = sc.upd_rhs[0] ? rrn / sc.rr[0] : 0.0;
+// Second step (rrn = |r_{k+1}|^2): beta, beta_i, the convergence of every
+// shift, the residual-replacement request and the count of columns still above
+// the precision-switch residual.
+template <int BC, int NT>
+__device__ void s2_tile(int j0, double rrn, const Scal &sc, const ShiftParams &sp, int B, double tol2, double delta2,
+                        double theta2, double *sm) {
+    __shared__ int any[BC]; // some shift is active
+    const int t = threadIdx.x;
+    if (t < BC) {
+        const int j = j0 + t;
+        if (j == 0) {
+            if (sc.hist) {
+                int it = sc.iter_counter[0];
+                if (it < sc.hist_len) sc.hist[sc.hist_len + it] = sc.upd_rhs[0] ? rrn / sc.rr[0] : 0.0;
+            }
+            sc.iter_counter[0] += 1;
         }
-        sc.iter_counter[0] += 1;
+        any[t] = 0;
+        sm[t] = rrn;
+        sm[BC + t] = sc.upd_rhs[j] ? rrn / sc.rr[j] : 0.0;
     }
-    const size_t row = (size_t)sc.slot[j] * sp.n * B + j;
-    sc.slot[j] += sc.slot_inc;
-    if (!sc.upd_rhs[j]) {
-        for (int i = 0; i < sp.n; ++i) { sc.hb[row + (size_t)i * B] = 1; sc.hz[row + (size_t)i * B] = 0; }
-        return;
-    }
-    double b = rrn / sc.rr[j];
-    sc.beta[j] = b;
-    int any = 0;
-    double bb = sc.bb[j];
-    for (int i = 0; i < sp.n; ++i) {
-        int ix = i * B + j;
-        const size_t hx = row + (size_t)i * B;
-        if (!sc.upd[ix]) {
-            any |= sc.act[ix];
-            sc.hb[hx] = 1;
-            sc.hz[hx] = 0;
-            continue;
+    __syncthreads();
+    constexpr int K = NT / BC;
+    if (t < K * BC) {
+        const int q = t % BC, j = j0 + q;
+        const size_t row = (size_t)sc.slot[j] * sp.n * B + j;
+        const bool on = sc.upd_rhs[j];
+        const double r2 = sm[q], b = sm[BC + q], bb = sc.bb[j];
+        for (int i = t / BC; i < sp.n; i += K) {
+            const int ix = i * B + j;
+            const size_t hx = row + (size_t)i * B;
+            if (!on || !sc.upd[ix]) {
+                if (on && sc.act[ix]) any[q] = 1;
+                sc.hb[hx] = 1;
+                sc.hz[hx] = 0;
+                continue;
+            }
+            double z = sc.zeta[ix], zn = sc.hz[hx];
+            double w = zn / z;
+            sc.hb[hx] = b * w * w;
+            sc.zeta_prev[ix] = z;
+            sc.zeta[ix] = zn;
+            int a = zn * zn * r2 > tol2 * bb;
+            sc.act[ix] = a;
+            if (a) any[q] = 1;
         }
-        double z = sc.zeta[ix], zn = sc.hz[hx];
-        double q = zn / z;
-        sc.hb[hx] = b * q * q;
-        sc.zeta_prev[ix] = z;
-        sc.zeta[ix] = zn;
-        int a = zn * zn * rrn > tol2 * bb;
-        sc.act[ix] = a;
-        any |= a;
     }
-    sc.alpha_prev[j] = sc.alpha[j];
-    sc.beta_prev[j] = b;
-    sc.rr[j] = rrn;
-    sc.iters[j] += 1;
-    sc.act_rhs[j] = any;
-    if (any) atomicAdd(&sc.flags[0], 1);
-    if (delta2 > 0 && rrn < delta2 * sc.rr_ref[j]) atomicOr(&sc.flags[1], 1);
-    if (any && rrn > theta2 * bb) atomicAdd(&sc.flags[3], 1); // still above the precision switch
+    __syncthreads();
+    if (t < BC) {
+        const int j = j0 + t;
+        sc.slot[j] += sc.slot_inc;
+        if (!sc.upd_rhs[j]) return;
+        const double bb = sc.bb[j];
+        sc.beta[j] = sm[BC + t];
+        sc.alpha_prev[j] = sc.alpha[j];
+        sc.beta_prev[j] = sm[BC + t];
+        sc.rr[j] = rrn;
+        sc.iters[j] += 1;
+        sc.act_rhs[j] = any[t];
+        if (any[t]) atomicAdd(&sc.flags[0], 1);
+        if (delta2 > 0 && rrn < delta2 * sc.rr_ref[j]) atomicOr(&sc.flags[1], 1);
+        if (any[t] && rrn > theta2 * bb) atomicAdd(&sc.flags[3], 1); // still above the precision switch
+    }
 }
 
 // What the lattice kernels A and B need for the scalar step of an RHS tile.
@@ -311,7 +341,7 @@ __device__ __forceinline__ void fuse_step1(const Fuse &f, int l, const double *p
     if (!f.count || !last_block_of_tile(f.count, G, threadIdx.x < BC)) return;
     const double tt = tile_sum<BC, NT>(part_t, prow, G, sm);
     const double pp = tile_sum<BC, NT>(part_p, prow, G, sm);
-    if (threadIdx.x < BC) s1_column(blockIdx.y * BC + threadIdx.x, tt, pp, f.sc, f.sp[l], f.B);
+    s1_tile<BC, NT>(blockIdx.y * BC, tt, pp, f.sc, f.sp[l], f.B, sm);
 }
 // end of lattice kernel B: the tile's last block runs the second scalar step
 template <int BC, int NT>
@@ -319,8 +349,7 @@ __device__ __forceinline__ void fuse_step2(const Fuse &f, int l, const double *p
                                            double *sm) {
     if (!f.count || !last_block_of_tile(f.count, G, threadIdx.x < BC)) return;
     const double rr = tile_sum<BC, NT>(part_r, prow, G, sm);
-    if (threadIdx.x < BC)
-        s2_column(blockIdx.y * BC + threadIdx.x, rr, f.sc, f.sp[l], f.B, f.tol2, f.delta2, f.theta2);
+    s2_tile<BC, NT>(blockIdx.y * BC, rr, f.sc, f.sp[l], f.B, f.tol2, f.delta2, f.theta2, sm);
 }
 
 // ------------------------------------------------------------------ lattice kernels
@@ -782,6 +811,213 @@ __device__ __forceinline__ void update_p_tiles(int bx, int tpb, int V, size_t ti
     }
 }
 
+// ------------------------------------------------------------------ FP64 iterations
+// SMPQ_FP64: p, t and r in block fixed point (bfp.cuh), one thread per site and
+// column.  Bound by the integer pipe: about 6400 (A) and 7000 (B) cycles a warp;
+// in FP64 arithmetic the pair took 46.7 + 48 ms for 3072 sources on 8^3x16, and
+// a small lattice's 24 blocks of 256 threads as long as a large one's.
+template <int BC>
+__global__ void __launch_bounds__(BfMap<BC>::THREADS)
+    k_init_bf(Geom g, Source src, BFF r, BFF p, double *part, int G) {
+    typedef BfMap<BC> TM;
+    __shared__ double sm[2 * TM::THREADS];
+    const int jj = threadIdx.x % BC, chunk = blockIdx.y, j = chunk * BC + jj;
+    const size_t base = (size_t)chunk * 12 * g.V * BC + jj, ebase = (size_t)chunk * g.V * BC + jj;
+    const BfOff<BC> off{g.V};
+    const int s = blockIdx.x * TM::SPB + threadIdx.x / BC;
+    double acc = 0;
+    if (s < g.V) {
+        double2 b[12];
+        bfc v[12];
+        int e;
+        bool wide;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            b[c] = source_at<BC>(src, g.V, s, c, j, base + ((size_t)s * 12 + c) * BC);
+            acc += b[c].x * b[c].x + b[c].y * b[c].y;
+        }
+        bf_from_double(b, v, e, wide);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            r.v[base + off(s, c)] = v[c];
+            p.v[base + off(s, c)] = v[c];
+        }
+        r.e[ebase + off.exp(s)] = e;
+        p.e[ebase + off.exp(s)] = e;
+    }
+    const double sum = block_sum<BC, TM::THREADS>(acc, sm);
+    if (threadIdx.x < BC) part[((size_t)chunk * G + blockIdx.x) * BC + threadIdx.x] = sum;
+}
+
+// t = D_W p; partials |t|^2, |p|^2
+template <int BC, bool M>
+__global__ void __launch_bounds__(BfMap<BC>::THREADS, BfMap<BC>::BLOCKS)
+    k_apply_a_bf(Lats L, BFF p, BFF t, BfScal kappa, double *part_t, double *part_p, int tpb, Fuse f) {
+    typedef BfMap<BC> TM;
+    __shared__ double sm[2 * TM::THREADS];
+    const int l = lat_index<M>(L);
+    const Lat &la = L.l[l];
+    if ((int)blockIdx.x >= la.G) return;
+    const Geom &g = la.g;
+    const int G = la.G, cl = blockIdx.y - la.chunk0;
+    const size_t prow = la.p0 + (size_t)cl * G;
+    const int jj = threadIdx.x % BC;
+    const size_t base = la.f0 + (size_t)cl * 12 * g.V * BC + jj, ebase = la.f0 / 12 + (size_t)cl * g.V * BC + jj;
+    const BfOff<BC> off{g.V};
+    const int ntiles = (g.V + TM::SPB - 1) / TM::SPB;
+    const int one = opaque_one();
+    double at = 0, ap = 0;
+    for (int tile = blockIdx.x * tpb, tend = min(ntiles, tile + tpb); tile < tend; ++tile) {
+        const int s = tile * TM::SPB + threadIdx.x / BC;
+        if (s >= g.V) continue;
+        bfc acc[12], own[12];
+        int eown, eref, e;
+        bf_wilson<false>(g, (const int4 *)la.U, p.v + base, p.e + ebase, off, s, one, acc, eown, eref);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) own[c] = p.v[base + off(s, c)];
+        ap += bf_norm2(own, eown, one);
+        bf_dw(own, eown, acc, eref, kappa, eown + 2, one, acc, e);
+        bf_normalise(acc, e);
+        at += bf_norm2(acc, e, one);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) t.v[base + off(s, c)] = acc[c];
+        t.e[ebase + off.exp(s)] = e;
+    }
+    const double s1 = block_sum<BC, TM::THREADS>(at, sm);
+    const double s2 = block_sum<BC, TM::THREADS>(ap, sm);
+    if (threadIdx.x < BC) {
+        part_t[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
+        part_p[(prow + blockIdx.x) * BC + threadIdx.x] = s2;
+    }
+    fuse_step1<BC, TM::THREADS>(f, l, part_t, part_p, prow, G, sm);
+}
+
+// r -= alpha (D_W^dag t + s0 p); partial |r|^2
+template <int BC, bool M>
+__global__ void __launch_bounds__(BfMap<BC>::THREADS, BfMap<BC>::BLOCKS)
+    k_apply_b_bf(Lats L, BFF t, BFF p, BFF r, const double *__restrict__ alpha, BfScal kappa, double *part_r, int tpb,
+                 Fuse f) {
+    typedef BfMap<BC> TM;
+    __shared__ double sm[2 * TM::THREADS];
+    const int l = lat_index<M>(L);
+    const Lat &la = L.l[l];
+    if ((int)blockIdx.x >= la.G) return;
+    const Geom &g = la.g;
+    const int G = la.G, cl = blockIdx.y - la.chunk0;
+    const size_t prow = la.p0 + (size_t)cl * G;
+    const int jj = threadIdx.x % BC, j = blockIdx.y * BC + jj;
+    const size_t base = la.f0 + (size_t)cl * 12 * g.V * BC + jj, ebase = la.f0 / 12 + (size_t)cl * g.V * BC + jj;
+    const BfOff<BC> off{g.V};
+    const int ntiles = (g.V + TM::SPB - 1) / TM::SPB;
+    const int one = opaque_one();
+    const BfScal s0 = bf_scal(la.s0), a = bf_scal(alpha[j]);
+    double ar = 0;
+    for (int tile = blockIdx.x * tpb, tend = min(ntiles, tile + tpb); tile < tend; ++tile) {
+        const int s = tile * TM::SPB + threadIdx.x / BC;
+        if (s >= g.V) continue;
+        bfc acc[12], own[12];
+        int eown, eref, eu;
+        bf_wilson<true>(g, (const int4 *)la.U, t.v + base, t.e + ebase, off, s, one, acc, eown, eref);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) own[c] = t.v[base + off(s, c)];
+        // the unit of A p = D_W^dag t + s0 p: its last term takes part in the choice
+        const int ep = p.e[ebase + off.exp(s)], ew = ep + s0.e + 64;
+        bf_dw(own, eown, acc, eref, kappa, max(eown + 3, ew + 1), one, acc, eu);
+        const int nw = eu - ew;
+        // r - alpha A p
+        int er = r.e[ebase + off.exp(s)];
+        const int ez = eu + a.e + 64, em = max(ez, er + 2), nz = em - ez, nr = em - er;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const size_t o = base + off(s, c);
+            const bfc pv = p.v[o], rv = r.v[o];
+            const long long x = acc[c].x + bf_shr(bf_mul(pv.x, s0, one), nw),
+                            y = acc[c].y + bf_shr(bf_mul(pv.y, s0, one), nw);
+            acc[c] = {bf_shr(rv.x, nr) - bf_shr(bf_mul(x, a, one), nz),
+                      bf_shr(rv.y, nr) - bf_shr(bf_mul(y, a, one), nz)};
+        }
+        er = max(eu, max(er, ep)) >= BF_BAD / 2 || a.e >= BF_BAD / 2 ? BF_BAD : em;
+        bf_normalise(acc, er);
+        ar += bf_norm2(acc, er, one);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) r.v[base + off(s, c)] = acc[c];
+        r.e[ebase + off.exp(s)] = er;
+    }
+    const double s1 = block_sum<BC, TM::THREADS>(ar, sm);
+    if (threadIdx.x < BC) part_r[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
+    fuse_step2<BC, TM::THREADS>(f, l, part_r, prow, G, sm);
+}
+
+// Launch YP of an FP64 iteration: r on the support into the history (as
+// doubles), p = r + beta p and, with x64, first x64 += alpha p on the lattice
+// (x64 in the tile layout).  tpb tiles of BfMap per block.
+template <int BC, bool M>
+__global__ void __launch_bounds__(BfMap<BC>::THREADS, 640 / BfMap<BC>::THREADS)
+    k_yp_bf(Lats L, int tpb, const int *__restrict__ rhs_class, BFF r, double2 *__restrict__ h, size_t stride, Scal sc,
+            BFF p, double2 *__restrict__ x64) {
+    typedef BfMap<BC> TM;
+    const int l = lat_index<M>(L);
+    const Lat &la = L.l[l];
+    const int cl = blockIdx.y - la.chunk0, V = la.g.V;
+    const int jj = threadIdx.x % BC, j = blockIdx.y * BC + jj;
+    if (!sc.upd_rhs[j]) return;
+    const size_t base = la.f0 + (size_t)cl * 12 * V * BC + jj, ebase = la.f0 / 12 + (size_t)cl * V * BC + jj;
+    const BfOff<BC> off{V};
+    if ((int)blockIdx.x < la.Gs) {
+        const int cls = rhs_class[j];
+        if (cls < 0) return;
+        double2 *o = h + la.sup0 + (size_t)(sc.slot[j] - 1) * stride + (size_t)cl * 12 * la.n_sup * BC + jj;
+        const int nt = (la.n_sup + TM::SPB - 1) / TM::SPB;
+        for (int tile = blockIdx.x * tpb, tend = min(nt, tile + tpb); tile < tend; ++tile) {
+            const int k = tile * TM::SPB + threadIdx.x / BC;
+            if (k >= la.n_sup) continue;
+            const int site = la.supsite ? la.supsite[(size_t)cls * la.n_sup + k] : k;
+            const int e = r.e[ebase + off.exp(site)];
+            bfc v[12];
+#pragma unroll
+            for (int c = 0; c < 12; ++c) v[c] = r.v[base + off(site, c)];
+#pragma unroll
+            for (int c = 0; c < 12; ++c)
+                o[((size_t)k * 12 + c) * BC] = make_double2(bf_double(v[c].x, e), bf_double(v[c].y, e));
+        }
+        return;
+    }
+    const int bx = blockIdx.x - la.Gs;
+    if (bx >= la.G) return;
+    const int nt = (V + TM::SPB - 1) / TM::SPB;
+    const int one = opaque_one();
+    const BfScal b = bf_scal(sc.beta[j]);
+    const double al = sc.alpha[j];
+    for (int tile = bx * tpb, tend = min(nt, tile + tpb); tile < tend; ++tile) {
+        const int s = tile * TM::SPB + threadIdx.x / BC;
+        if (s >= V) continue;
+        const int er = r.e[ebase + off.exp(s)];
+        int ep = p.e[ebase + off.exp(s)];
+        const int ez = ep + b.e + 64, em = max(ez, er + 2), nz = em - ez, nr = em - er;
+        bfc v[12], rv[12];
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            rv[c] = r.v[base + off(s, c)];
+            v[c] = p.v[base + off(s, c)];
+        }
+        if (x64)
+#pragma unroll
+            for (int c = 0; c < 12; ++c) {
+                double2 &x = x64[base + ((size_t)s * 12 + c) * BC];
+                x = make_double2(fma(al, bf_double(v[c].x, ep), x.x), fma(al, bf_double(v[c].y, ep), x.y));
+            }
+#pragma unroll
+        for (int c = 0; c < 12; ++c)
+            v[c] = {bf_shr(rv[c].x, nr) + bf_shr(bf_mul(v[c].x, b, one), nz),
+                    bf_shr(rv[c].y, nr) + bf_shr(bf_mul(v[c].y, b, one), nz)};
+        ep = max(er, ep) >= BF_BAD / 2 || b.e >= BF_BAD / 2 ? BF_BAD : em;
+        bf_normalise(v, ep);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) p.v[base + off(s, c)] = v[c];
+        p.e[ebase + off.exp(s)] = ep;
+    }
+}
+
 // ------------------------------------------------------------------ half-storage iterations
 // SMPQ_FP16N / SMPQ_BF16N: the FP32 path (FP64 reliable updates, FP32 r, x_lo
 // and shifted directions) with p and t -- the input and output of D_W --
@@ -1091,14 +1327,6 @@ __global__ void __launch_bounds__(TileMap<BC, 2>::THREADS, 2)
 //
 // slot q of a lattice: H[q * stride + element], elements [tile][n_sup][12][BC]
 
-// exact float -> double without the FP64 pipe (a conversion there costs 66 cycles a warp)
-__device__ __forceinline__ double exact_d(float f) {
-    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
-    if ((e == 0 && (u << 1) != 0) || e == 0x7f800000u) return (double)f; // subnormal, infinity, NaN
-    const bool z = e == 0;
-    return __hiloint2double((int)((u & 0x80000000u) | (z ? 0u : ((u & 0x7fffffffu) >> 3) + 0x38000000u)),
-                            (int)(z ? 0u : u << 29));
-}
 __device__ __forceinline__ double2 hist_value(double2 v) { return v; }
 __device__ __forceinline__ double2 hist_value(float2 v) { return make_double2(exact_d(v.x), exact_d(v.y)); }
 __device__ __forceinline__ double2 hist_value(df64c v) {
@@ -1770,7 +1998,8 @@ template <int BC> struct Solve {
             nsupf += (size_t)sp.B * 12 * sp.n_sup;
             // partial rows per tile: the most blocks any launch has per tile (the
             // D_W launches at one tile per block have nt1; the support kernels Gs1)
-            npart += (size_t)nch[l] * std::max(nt1[l], Gs1[l]) * BC;
+            const int ntb = (V[l] + BfMap<BC>::SPB - 1) / BfMap<BC>::SPB;
+            npart += (size_t)nch[l] * std::max(std::max(nt1[l], ntb), Gs1[l]) * BC;
             sph[l] = in[l].sp;
         }
         tpb_hi = std::max(1, in[0].spec->tpb_hi > 0 ? in[0].spec->tpb_hi : TPB);
@@ -1872,9 +2101,9 @@ template <int BC> struct Solve {
     }
     // the lattice table of launch YP: support blocks, then lattice blocks (one
     // column per thread, *tpb tiles per block: as many as leave each SM several blocks)
-    Lats lats_yp(int *gx, int *tpb) const {
+    Lats lats_yp(int spb, int *gx, int *tpb) const {
         size_t tiles = 0;
-        for (int l = 0; l < nl; ++l) tiles += (size_t)nch[l] * nt1[l];
+        for (int l = 0; l < nl; ++l) tiles += (size_t)nch[l] * ((V[l] + spb - 1) / spb);
         *tpb = TPB;
         while (*tpb > 1 && tiles / *tpb < 2048) *tpb /= 2;
         Lats L{};
@@ -1885,8 +2114,8 @@ template <int BC> struct Solve {
             a.g = in[l].ctx->geom;
             a.f0 = (long long)f0[l];
             a.chunk0 = ch0[l];
-            const int nst = (in[l].spec->n_sup + TileMap<BC>::SPB - 1) / TileMap<BC>::SPB;
-            a.G = (nt1[l] + *tpb - 1) / *tpb;
+            const int nst = (in[l].spec->n_sup + spb - 1) / spb;
+            a.G = ((V[l] + spb - 1) / spb + *tpb - 1) / *tpb;
             a.Gs = shifts ? (nst + *tpb - 1) / *tpb : 0;
             a.n_sup = in[l].spec->n_sup;
             a.supsite = in[l].spec->d_supsite;
@@ -1927,6 +2156,12 @@ template <int BC> struct Solve {
         }
         (hi ? ctx->prof_a_hi_n : ctx->prof_a_n) += n;
         (hi ? ctx->prof_b_hi_n : ctx->prof_b_n) += n;
+    }
+
+    // a block-fixed-point field of this solve passed through a double2 pointer, from element o on
+    BFF bfield(void *f, size_t o = 0) const {
+        bfc *v = (bfc *)f;
+        return BFF{v + o, (int *)(v + nfield) + o / 12};
     }
 
     // a half-format field of this solve passed through a float2 pointer
@@ -2069,12 +2304,18 @@ template <int BC> struct Solve {
               bool replace_mid = true) {
         typedef typename cplx_t<T>::type C;
         constexpr bool half = !std::is_void<HT>::value;
+        constexpr bool fixed_point = std::is_same<T, double>::value; // p, t, r through double2 pointers
         const int TH = TileMap<BC>::THREADS;
         const bool hi = sizeof(T) != sizeof(float); // FP64 or float-float iterations
         const bool multi = nl > 1;
         // kernel shape of the D_W launches (the autotuner's choice): tiles per
         // block, per phase, and for the FP32 kernels one or two columns per thread
-        const int tpb = hi ? tpb_hi : tpb_lo;
+        int tpb = hi ? tpb_hi : tpb_lo;
+        if (fixed_point && in[0].spec->tpb_hi == 0) { // no tuned shape: several blocks for each SM
+            size_t tiles = 0;
+            for (int l = 0; l < nl; ++l) tiles += (size_t)nch[l] * ((V[l] + BfMap<BC>::SPB - 1) / BfMap<BC>::SPB);
+            while (tpb > 1 && tiles / tpb < 2048) tpb /= 2;
+        }
         const bool two_cols = std::is_same<T, float>::value && !half && nr == 2 && BC % 2 == 0 && !multi;
         constexpr bool can_stage = std::is_same<T, float>::value && !half && BC >= 12;
         constexpr bool can_stage_df = std::is_same<T, df64>::value && BC >= 12;
@@ -2113,8 +2354,9 @@ template <int BC> struct Solve {
         // and the one-column lattice kernels
         {
             size_t rows = 0;
+            const int spb = fixed_point ? BfMap<BC>::SPB : TileMap<BC>::SPB;
             for (int l = 0; l < nl; ++l)
-                rows += (size_t)nch[l] * std::max((nt1[l] + tpb - 1) / tpb, G1[l]);
+                rows += (size_t)nch[l] * std::max(((V[l] + spb - 1) / spb + tpb - 1) / tpb, G1[l]);
             if (rows * BC > npart)
                 return set_err(ctx, SMPQ_EINVAL, "internal: launch shape exceeds the partial-sum buffers");
         }
@@ -2124,13 +2366,18 @@ template <int BC> struct Solve {
                 const Geom &g = in[l].ctx->geom;
                 const size_t o = f0[l];
                 double *pl = part0 + p0[l] * BC;
-                if constexpr (half)
+                int G = G1[l];
+                if constexpr (fixed_point) {
+                    G = (V[l] + BfMap<BC>::SPB - 1) / BfMap<BC>::SPB;
+                    k_init_bf<BC><<<dim3(G, nch[l]), BfMap<BC>::THREADS, 0, st>>>(g, srcl[l], bfield(r, o), bfield(p, o),
+                                                                                 pl, G);
+                } else if constexpr (half)
                     k_init_h<HT, BC><<<grid, TH, 0, st>>>(g, srcl[l], (float2 *)r + o, hfield_at<HT>(p, o),
                                                           (float2 *)xlo + o, xhi + o, pl, G1[l]);
                 else
                     k_init<T, BC><<<grid, TH, 0, st>>>(g, srcl[l], r + o, p + o, xlo ? xlo + o : nullptr,
                                                        xhi ? xhi + o : nullptr, pl, G1[l]);
-                s_init<<<Bl[l], SCAL_THREADS, 0, st>>>(B, BC, G1[l], pl, scal_of(l), sph[l], sqrt(tol2));
+                s_init<<<Bl[l], SCAL_THREADS, 0, st>>>(B, BC, G, pl, scal_of(l), sph[l], sqrt(tol2));
                 ctx->launches += 2;
             }
         }
@@ -2138,7 +2385,7 @@ template <int BC> struct Solve {
         const Fuse f1{count, sc, spd, B, 0.0, 0.0, 0.0};
         const Fuse f2{count, sc, spd, B, tol2, delta2, theta2};
         int gyp, tyy;
-        const Lats Lyp = lats_yp(&gyp, &tyy);
+        const Lats Lyp = lats_yp(fixed_point ? BfMap<BC>::SPB : TileMap<BC>::SPB, &gyp, &tyy);
         C *hbase = shifts ? (C *)ctx->ws[W_HIST].p : nullptr;
         const dim3 gridyp(gyp, nchunk);
         const int *rhs_class = in[0].spec->d_rhs_class;
@@ -2187,6 +2434,25 @@ template <int BC> struct Solve {
             auto launch = [&](auto nr_c, auto m) {
                 constexpr int NR = decltype(nr_c)::value;
                 constexpr bool M = decltype(m)::value;
+                if constexpr (fixed_point) {
+                    if constexpr (NR == 1) {
+                        int gx;
+                        const Lats Ld = lats_dw<T>(BfMap<BC>::SPB, tpb, &gx);
+                        const BFF bp = bfield(p), bt = bfield(t), br = bfield(r);
+                        const BfScal ks = bf_scal(kd);
+                        constexpr int THB = BfMap<BC>::THREADS;
+                        if (prof) cudaEventRecord(ctx->prof_ev[4 * k], st);
+                        k_apply_a_bf<BC, M><<<dim3(gx, nchunk), THB, 0, st>>>(Ld, bp, bt, ks, part0, part1, tpb, f1);
+                        if (prof) cudaEventRecord(ctx->prof_ev[4 * k + 1], st);
+                        if (prof) cudaEventRecord(ctx->prof_ev[4 * k + 2], st);
+                        k_apply_b_bf<BC, M><<<dim3(gx, nchunk), THB, 0, st>>>(Ld, bt, bp, br, sc.alpha, ks, part2, tpb,
+                                                                              f2);
+                        if (prof) cudaEventRecord(ctx->prof_ev[4 * k + 3], st);
+                        k_yp_bf<BC, M><<<gridyp, THB, 0, st>>>(Lyp, tyy, rhs_class, br, (double2 *)hbase, nsupf, sc, bp,
+                                                               (double2 *)xacc);
+                    }
+                    return;
+                }
                 if constexpr (can_stage && NR == 1) {
                     if (staged) {
                         int gx;
@@ -2223,7 +2489,7 @@ template <int BC> struct Solve {
                         return;
                     }
                 }
-                if constexpr (NR == 1 || (std::is_same<T, float>::value && BC % 2 == 0 && !M)) {
+                if constexpr (!fixed_point && (NR == 1 || (std::is_same<T, float>::value && BC % 2 == 0 && !M))) {
                     typedef TileMap<BC, NR> TMN;
                     int gx;
                     const Lats Ld = lats_dw<T>(TMN::SPB, tpb, &gx);
@@ -2244,6 +2510,8 @@ template <int BC> struct Solve {
         };
         // residual replacement, lattice by lattice: x_hi += x_lo, r = b - (A + s0) x_hi in float-float
         auto reliable = [&]() {
+            if constexpr (fixed_point) return; // (no residual replacement in FP64)
+            else {
             const df64 kdf(ctx->opt.kappa);
             Fuse none{};
             for (int l = 0; l < nl; ++l) {
@@ -2277,6 +2545,7 @@ template <int BC> struct Solve {
                                                                                    sc.act_rhs + j0[l]);
                     ctx->launches += 1;
                 }
+            }
             }
         };
         if (fixed > 0) {
@@ -2471,9 +2740,10 @@ template <int BC> struct Solve {
         const int prec = lats[0].spec->prec;
         cudaEventRecord(ctx->ev1, S.st);
         if (prec == SMPQ_FP64) {
-            if ((rc = ensure(ctx, ws[W_P], nf * sizeof(double2)))) return rc;
-            if ((rc = ensure(ctx, ws[W_T], nf * sizeof(double2)))) return rc;
-            if ((rc = ensure(ctx, ws[W_R], nf * sizeof(double2)))) return rc;
+            const size_t fb = nf * sizeof(bfc) + nf / 12 * sizeof(int);
+            if ((rc = ensure(ctx, ws[W_P], fb))) return rc;
+            if ((rc = ensure(ctx, ws[W_T], fb))) return rc;
+            if ((rc = ensure(ctx, ws[W_R], fb))) return rc;
             if (shifts && (rc = ensure(ctx, ws[W_Y], S.nsupf * sizeof(double2)))) return rc;
             S.y = shifts ? (double2 *)ws[W_Y].p : nullptr;
             if ((rc = S.alloc_x64())) return rc;
@@ -2630,6 +2900,27 @@ float time_pair(smpq_ctx *ctx, int B, int tpb, int reps, void *buf, double *part
     });
 }
 
+// the FP64 pair (block fixed point)
+template <int BC> float time_pair_bf(smpq_ctx *ctx, int B, int tpb, int reps, void *buf, double *part, double *alpha) {
+    typedef BfMap<BC> TM;
+    const int V = ctx->V, nchunk = B / BC;
+    const int GN = ((V + TM::SPB - 1) / TM::SPB + tpb - 1) / tpb;
+    const size_t nf = (size_t)B * 12 * V;
+    bfc *v = (bfc *)buf;
+    int *e = (int *)(v + 3 * nf);
+    const BFF p{v, e}, t{v + nf, e + nf / 12}, r{v + 2 * nf, e + 2 * (nf / 12)};
+    const Lats L = lats_single(ctx, ctx->Ubf.p, GN);
+    const BfScal ks = bf_scal(ctx->opt.kappa);
+    cudaStream_t st = ctx->stream;
+    const dim3 gridn(GN, nchunk);
+    Fuse none{};
+    return time_launches(ctx, reps, [&]() {
+        k_apply_a_bf<BC, false><<<gridn, TM::THREADS, 0, st>>>(L, p, t, ks, part, part + (size_t)nchunk * GN * BC, tpb,
+                                                               none);
+        k_apply_b_bf<BC, false><<<gridn, TM::THREADS, 0, st>>>(L, t, p, r, alpha, ks, part, tpb, none);
+    });
+}
+
 // the FP32 pair with staged neighbours (one column per thread); -1 if a
 // staging wait ran out (*err, zero on entry)
 template <int BC>
@@ -2719,7 +3010,7 @@ float time_pair_half(smpq_ctx *ctx, int B, int tpb, int reps, void *buf, double 
 template <int BC> float time_kind(smpq_ctx *ctx, int kind, int B, int tpb, int nr, int reps, void *buf, double *part,
                                   double *alpha, int *err) {
     switch (kind) {
-    case 0: return time_pair<double, BC, 1>(ctx, B, tpb, reps, buf, part, alpha);
+    case 0: return time_pair_bf<BC>(ctx, B, tpb, reps, buf, part, alpha);
     case 1:
         return nr == 2 ? time_pair<float, BC, 2>(ctx, B, tpb, reps, buf, part, alpha)
                        : time_pair<float, BC, 1>(ctx, B, tpb, reps, buf, part, alpha);

@@ -39,6 +39,7 @@ struct smpq_ctx {
     int dims[4] = {0, 0, 0, 0};
     int V = 0;
     Buf U64, U32, Udf; // FP64, FP32 and float-float copies of the links
+    Buf Ubf;           // the links as 64-bit integers (bfp.cuh)
     Buf d_err;         // int: set by a staged D_W whose staging wait ran out
     Buf Uh16, Ub16;    // rows 0 and 1 of the links in FP16 and BF16 (reconstruct-12)
 
@@ -110,7 +111,7 @@ int colour_sites_host(const int dims[4], int r, int mode, std::vector<int> &colo
 
 // ---------------------------------------------------------------- kernel launchers
 // dslash.cu
-void launch_pack_links(const double *U_aos, double *U64, float *U32, void *Udf, int V, cudaStream_t st);
+void launch_pack_links(const double *U_aos, double *U64, float *U32, void *Udf, void *Ubf, int V, cudaStream_t st);
 void launch_su3_check(const double *U64, int V, double *dev_maxerr, cudaStream_t st);
 // convert ABI spinors [V][12][B] (FP64) <-> internal tiled layout of precision T
 template <typename T> void launch_to_tiled(const double *in, void *out, int V, int B, int BC, cudaStream_t st);
@@ -118,6 +119,16 @@ template <typename T> void launch_from_tiled(const void *in, double *out, int V,
 // out = D_W in (or D_W^dag), tiled layout, no reductions
 template <typename T> void launch_dslash(const Geom &g, const void *U, const void *in, void *out, int B, int BC,
                                          int dagger, double kappa, cudaStream_t st);
+
+// D_W on the caller's layout [V][12][B]: in converted to a block-fixed-point
+// field (bf_field_bytes) and then out (not overlapping in) = D_W in; the FP32 one
+// takes a field of 12 V B float2 (out may be in)
+size_t bf_field_bytes(int V, int B);
+void launch_abi_to_bf(const double *in, void *field, int V, int B, cudaStream_t st);
+void launch_dslash_bf(const Geom &g, const void *Ubf, const void *U64, const void *field, const double *in,
+                      double *out, int B, int dagger, double kappa, cudaStream_t st);
+void launch_dslash_fp32_abi(const Geom &g, const void *U, const double *in, void *field, double *out, int B,
+                            int dagger, double kappa, cudaStream_t st);
 
 // half.cu : SMPQ_FP16N / SMPQ_BF16N storage for the stand-alone D_W.  A half
 // field of B columns is one buffer of half_field_bytes(V, B): the components

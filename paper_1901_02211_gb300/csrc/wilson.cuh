@@ -64,18 +64,19 @@ template <> struct Cols<float2, 2> {
 template <typename T, int MU, int SG, bool BACK, int BC, int NR = 1>
 __device__ __forceinline__ void hop_one(const typename cplx_t<T>::type *__restrict__ U,
                                         const typename cplx_t<T>::type *__restrict__ in, int Vf, int Vl, int nb,
-                                        int ls, bool flip, typename cplx_t<T>::type acc[12][NR]) {
+                                        int ls, bool flip, typename cplx_t<T>::type acc[12][NR], int stride = 0) {
     typedef typename cplx_t<T>::type C;
-    const C *q = in + (size_t)nb * (12 * BC); // the 12 components of a site are BC apart
+    const int bc = BC ? BC : stride; // BC = 0: the column stride is only known at run time
+    const C *q = in + (size_t)nb * 12 * bc; // the 12 components of a site are bc apart
     // project colour by colour: only the 4 spin components of one colour are live
     C h[2][3][NR];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         C p0[NR], p1[NR], p2[NR], p3[NR];
-        Cols<C, NR>::load(q + a * BC, p0);
-        Cols<C, NR>::load(q + (3 + a) * BC, p1);
-        Cols<C, NR>::load(q + (6 + a) * BC, p2);
-        Cols<C, NR>::load(q + (9 + a) * BC, p3);
+        Cols<C, NR>::load(q + a * bc, p0);
+        Cols<C, NR>::load(q + (3 + a) * bc, p1);
+        Cols<C, NR>::load(q + (6 + a) * bc, p2);
+        Cols<C, NR>::load(q + (9 + a) * bc, p3);
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             C s0, s1;
@@ -146,7 +147,7 @@ template <typename T, int MU, bool DAG, int BC, int NR>
 __device__ __forceinline__ void hop_dir(const Geom &g, const SiteCoords &xc,
                                         const typename cplx_t<T>::type *__restrict__ U,
                                         const typename cplx_t<T>::type *__restrict__ in, int s,
-                                        typename cplx_t<T>::type acc[12][NR]) {
+                                        typename cplx_t<T>::type acc[12][NR], int stride) {
     const int n = g.n[MU], st = g.stride[MU], c = xc.x[MU];
     const bool top = c == n - 1, bot = c == 0;
     const int nf = top ? s - (n - 1) * st : s + st;
@@ -154,10 +155,10 @@ __device__ __forceinline__ void hop_dir(const Geom &g, const SiteCoords &xc,
     const bool ff = top && g.bcf[MU] < 0;
     const bool fb = bot && g.bcf[MU] < 0;
     // forward: (1 - g) U(x) psi(x+mu)   [DAG: (1 + g)]
-    hop_one<T, MU, DAG ? +1 : -1, false, BC, NR>(U, in, g.V, g.V, nf, s, ff, acc);
+    hop_one<T, MU, DAG ? +1 : -1, false, BC, NR>(U, in, g.V, g.V, nf, s, ff, acc, stride);
     SMPQ_HOP_BARRIER();
     // backward: (1 + g) U(x-mu)^dag psi(x-mu)   [DAG: (1 - g)]
-    hop_one<T, MU, DAG ? -1 : +1, true, BC, NR>(U, in, g.V, g.V, nbk, nbk, fb, acc);
+    hop_one<T, MU, DAG ? -1 : +1, true, BC, NR>(U, in, g.V, g.V, nbk, nbk, fb, acc, stride);
     SMPQ_HOP_BARRIER();
 }
 
@@ -166,17 +167,17 @@ __device__ __forceinline__ void hop_dir(const Geom &g, const SiteCoords &xc,
 template <typename T, bool DAG, int BC, int NR = 1>
 __device__ __forceinline__ void wilson_hop(const Geom &g, const typename cplx_t<T>::type *__restrict__ U,
                                            const typename cplx_t<T>::type *__restrict__ in, int s,
-                                           typename cplx_t<T>::type acc[12][NR]) {
+                                           typename cplx_t<T>::type acc[12][NR], int stride = 0) {
     typedef typename cplx_t<T>::type C;
 #pragma unroll
     for (int c = 0; c < 12; ++c)
 #pragma unroll
         for (int r = 0; r < NR; ++r) acc[c][r] = mkc<C>(0, 0);
     const SiteCoords xc(g, s);
-    hop_dir<T, 0, DAG, BC, NR>(g, xc, U, in, s, acc);
-    hop_dir<T, 1, DAG, BC, NR>(g, xc, U, in, s, acc);
-    hop_dir<T, 2, DAG, BC, NR>(g, xc, U, in, s, acc);
-    hop_dir<T, 3, DAG, BC, NR>(g, xc, U, in, s, acc);
+    hop_dir<T, 0, DAG, BC, NR>(g, xc, U, in, s, acc, stride);
+    hop_dir<T, 1, DAG, BC, NR>(g, xc, U, in, s, acc, stride);
+    hop_dir<T, 2, DAG, BC, NR>(g, xc, U, in, s, acc, stride);
+    hop_dir<T, 3, DAG, BC, NR>(g, xc, U, in, s, acc, stride);
 }
 
 // ---------------------------------------------------------------- rolled variant
