@@ -147,26 +147,60 @@ void launch_pack_links12(const double *U_aos, void *Uh, void *Ub, int V, cudaStr
 }
 
 // ABI double[V][12][B][2] -> half format (tile BC); one thread per (site, rhs).
-// norm = FP32 copy of max |re|, |im|; stored value = component / norm.
+// norm n = FP32 copy of max |re|, |im|; stored value = component / n, rounded to
+// FP32 and then to the half format.  The quotients run on the FP32 and integer
+// pipes: v / 2^E = h + l (h its leading 24 bits, l the rest), 1 / n' by one
+// Newton step, q = h / n' with the exact remainder h - q n' + l added: about 2^-45
+// before the rounding to FP32 (as FP64 divisions of 20 instructions each,
+// 66 cycles a warp, they were 352 of 517 us for 96 columns of 8^3x16).  A
+// component outside 2^-70 .. 2^70 of n, or a norm that is not a normal finite
+// number, takes the FP64 division.
 template <typename HT>
-__global__ void to_half_kernel(const double2 *__restrict__ in, typename HT::h2 *__restrict__ out,
-                               float *__restrict__ nout, int V, int B, int BC) {
+__global__ void __launch_bounds__(128) to_half_kernel(const double2 *__restrict__ in,
+                                                      typename HT::h2 *__restrict__ out, float *__restrict__ nout,
+                                                      int V, int B, int BC) {
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (i >= (long)V * B) return;
     const int j = (int)(i % B), s = (int)(i / B);
     double2 v[12];
-    double mx = 0;
+    unsigned long long top = 0; // max |component|: non-negative doubles order like integers
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
         v[c] = in[((size_t)s * 12 + c) * B + j];
-        mx = fmax(mx, fmax(fabs(v[c].x), fabs(v[c].y)));
+        const unsigned long long m = 0x7fffffffffffffffull;
+        const unsigned long long x = __double_as_longlong(v[c].x) & m, y = __double_as_longlong(v[c].y) & m;
+        top = x > top ? x : top;
+        top = y > top ? y : top;
+    }
+    double mx = __longlong_as_double((long long)top);
+    if (top > 0x7ff0000000000000ull) { // a NaN somewhere: the largest of the others
+        mx = 0;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) mx = fmax(mx, fmax(fabs(v[c].x), fabs(v[c].y)));
     }
     const float n = (float)mx;
     const double dn = n > 0.f ? (double)n : 1.0;
+    const int ne = (__float_as_int(n) >> 23) & 0xff;
+    const bool plain = ne > 0 && ne < 255;
+    const float nm = __int_as_float((__float_as_int(n) & 0x007fffff) | 0x3f800000); // n / 2^E in [1, 2)
+    float rc = 1.f / nm;
+    rc = fmaf(fmaf(-nm, rc, 1.f), rc, rc);
     const size_t t = (size_t)(j / BC), jj = (size_t)(j % BC);
+    auto quotient = [&](double x) -> float {
+        const int hi = __double2hiint(x), lo = __double2loint(x);
+        const int e = ((hi >> 20) & 0x7ff) - 1023 - (ne - 127); // exponent of x / 2^E
+        if (((hi & 0x7fffffff) | lo) == 0) return __int_as_float(hi); // +-0
+        if (!plain || e < -70 || e > 70) return (float)(x / dn);
+        const float h = __int_as_float((hi & 0x80000000) | ((e + 127) << 23) |
+                                       (((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29)));
+        // the 29 bits below, times 2^(e - 52)
+        const float l = (float)(lo & 0x1fffffff) * __int_as_float((e - 52 + 127) << 23);
+        const float q = h * rc, r = fmaf(-q, nm, h) + (hi < 0 ? -l : l);
+        return fmaf(r, rc, q);
+    };
 #pragma unroll
     for (int c = 0; c < 12; ++c)
-        out[((t * V + s) * 12 + c) * BC + jj] = HT::pack(make_float2((float)(v[c].x / dn), (float)(v[c].y / dn)));
+        out[((t * V + s) * 12 + c) * BC + jj] = HT::pack(make_float2(quotient(v[c].x), quotient(v[c].y)));
     nout[(t * V + s) * BC + jj] = n;
 }
 
@@ -177,11 +211,19 @@ __global__ void from_half_kernel(const typename HT::h2 *__restrict__ in, const f
     if (i >= (long)V * B) return;
     const int j = (int)(i % B), s = (int)(i / B);
     const size_t t = (size_t)(j / BC), jj = (size_t)(j % BC);
-    const double n = nin[(t * V + s) * BC + jj];
+    const float n = nin[(t * V + s) * BC + jj];
+    // n * f exactly (24 x 11 bits): the FP32 product and its exact error, in one FP64
+    // addition (conversions and a multiplication there cost 66 cycles a warp each)
+    auto wide = [&](float f) {
+        const float p = n * f, a = fabsf(p);
+        if (!(a < 3e38f) || (a < 1e-25f && f != 0.f)) // (its error could be subnormal)
+            return (double)n * (double)f;
+        return exact_d(p) + exact_d(fmaf(n, f, -p));
+    };
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
         const float2 f = HT::f2(in[((t * V + s) * 12 + c) * BC + jj]);
-        out[((size_t)s * 12 + c) * B + j] = make_double2(n * (double)f.x, n * (double)f.y);
+        out[((size_t)s * 12 + c) * B + j] = make_double2(wide(f.x), wide(f.y));
     }
 }
 
@@ -247,15 +289,15 @@ void launch_dslash_half(int prec, const Geom &g, const void *U, const void *in, 
 
 void launch_to_half(int prec, const double *in, void *out, int V, int B, cudaStream_t st) {
     const long n = (long)V * B;
-    const unsigned nb = (unsigned)((n + 255) / 256);
+    const unsigned nb = (unsigned)((n + 127) / 128);
     const int BC = half_tile(B);
     const size_t ncomp = (size_t)V * 12 * B;
     if (prec == SMPQ_BF16N) {
         __nv_bfloat162 *o = (__nv_bfloat162 *)out;
-        to_half_kernel<B16><<<nb, 256, 0, st>>>((const double2 *)in, o, (float *)(o + ncomp), V, B, BC);
+        to_half_kernel<B16><<<nb, 128, 0, st>>>((const double2 *)in, o, (float *)(o + ncomp), V, B, BC);
     } else {
         __half2 *o = (__half2 *)out;
-        to_half_kernel<H16><<<nb, 256, 0, st>>>((const double2 *)in, o, (float *)(o + ncomp), V, B, BC);
+        to_half_kernel<H16><<<nb, 128, 0, st>>>((const double2 *)in, o, (float *)(o + ncomp), V, B, BC);
     }
 }
 
