@@ -56,9 +56,6 @@ CONFIG = "flux8x16"
 # = 8592, plus the epilogue (1368 for t = D_W p with norms, 1824 for the r update)
 DF64_OPS_A = 8592 + 1368
 DF64_OPS_B = 8592 + 1824
-# FP64 D_W: 1320 flop hopping + 24 (kappa scale) + 24 (norm) / + 72 (update and norm)
-FP64_FLOP_A = 1320 + 48
-FP64_FLOP_B = 1320 + 96
 R_MIN, MODE = 4, 0
 KAPPA = 0.21
 
@@ -299,12 +296,7 @@ def _kernel_table(prec, stats, V, B, peak_hbm, peak_kind, alu):
             k["alu"] = dict(achieved=ops / (ms / 1000.0) / 1e12, peak=pk, unit="T FP32 lane-ops/s",
                             frac=ops / (ms / 1000.0) / 1e12 / pk, algorithmic=ops,
                             peak_source="measured (smpq_alu_peak, packed FFMA2 probe)")
-        elif esz_k == 16 and "fp64_fma_per_s" in alu:  # native FP64
-            fl = V * B * (FP64_FLOP_A if key.startswith("k_apply_a") else FP64_FLOP_B)
-            pk = 2 * alu["fp64_fma_per_s"] / 1e12
-            k["alu"] = dict(achieved=fl / (ms / 1000.0) / 1e12, peak=pk, unit="TFLOP/s (FP64)",
-                            frac=fl / (ms / 1000.0) / 1e12 / pk, algorithmic=fl,
-                            peak_source="measured (smpq_alu_peak, DFMA probe, 2 flop each)")
+        # (FP64 iterations run in block fixed point on the integer pipe: bytes only)
         kern[key] = k
     return kern
 

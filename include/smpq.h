@@ -251,10 +251,11 @@ int smpq_dslash(smpq_ctx *ctx, const double *in, double *out, int B, int dagger,
 
 /* Average device time of one stand-alone D_W launch (the kernel behind
  * smpq_dslash, Sec. 2.1, Eq. 3) on B right-hand sides held in `precision`
- * (SMPQ_FP64, SMPQ_FP32, SMPQ_FP16N or SMPQ_BF16N), in the RHS tile the
- * library picks for B.  The input and output fields are scratch in the
- * context's workspace, set once to the byte 0x3F (finite values in every
- * format; the values do not change the work).  Two untimed launches, then
+ * (SMPQ_FP64: block fixed point, 64-bit integers with one exponent per site and
+ * rhs, written as doubles; SMPQ_FP32, SMPQ_FP16N or SMPQ_BF16N), in the RHS tile
+ * the library picks for B.  The input and output fields are scratch in the
+ * context's workspace, set once to the byte 0x3F (SMPQ_FP64: 0; finite values in
+ * every format; the values do not change the work).  Two untimed launches, then
  * `reps` (>= 1) launches back to back on the context's stream between two
  * CUDA events.  *ms (nullable): average milliseconds per launch; *bytes
  * (nullable): algorithmic bytes of one launch, V * B * (spinor bytes read +

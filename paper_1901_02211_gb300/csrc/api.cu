@@ -339,13 +339,17 @@ int compute_classes(smpq_ctx *ctx, const std::vector<int> &classes, double *q_re
         if (kind == 0 && ctx->lm_k > 0) per += (size_t)ctx->V * 12 * sizeof(double2); // projected source field
         long cap = (long)((0.6 * (double)(freeb + held)) / (double)per);
         cap = std::max(12L, cap - cap % 48);
-        // As few batches as the memory allows, of equal size, in whole 48-column
-        // tiles (972 sources: one batch of 1008; 960 and a second batch of which
-        // 948 columns were padding took twice as long); 24-column ones in FP64,
-        // whose kernels are as fast in them.  Up to 48 sources: as they are.
-        const long nb = (nrhs_total + cap - 1) / cap, tile = prec == SMPQ_FP64 ? 24 : 48;
-        B = (int)std::min<long>(cap, nrhs_total <= 48 ? nrhs_total
-                                                      : ((nrhs_total + nb - 1) / nb + tile - 1) / tile * tile);
+        // FP64: as few batches as the memory allows, of equal size, in 24-column
+        // tiles.  Else batches of whole 48-column tiles, the last one as long as
+        // its sources (972: 960 and 48 columns; the second padded to 960 as well
+        // took as long as the first).
+        if (prec == SMPQ_FP64 && nrhs_total > 48) {
+            const long nb = (nrhs_total + cap - 1) / cap;
+            B = (int)std::min<long>(cap, ((nrhs_total + nb - 1) / nb + 23) / 24 * 24);
+        } else {
+            B = (int)std::min<long>(nrhs_total, cap);
+            if (B > 48) B -= B % 48;
+        }
     }
     if (B > 1) B -= B % 12;
     if (B < 1) B = 1;
@@ -403,6 +407,9 @@ int compute_classes(smpq_ctx *ctx, const std::vector<int> &classes, double *q_re
     long long totit = 0;
     double worst = 0, solve_ms = 0, true_res = -1;
     for (int j0 = 0; j0 < nrhs_total; j0 += B) {
+        // a last batch of fewer sources: whole tiles of 48 that hold them
+        const int left = nrhs_total - j0, Bb = BC > 1 && B % 48 == 0 ? std::min(B, (left + 47) / 48 * 48) : B;
+        spec.B = Bb;
         for (int j = 0; j < B; ++j) {
             int g = j0 + j;
             int cl = g < nrhs_total ? classes[g / 12] : -1;
@@ -413,35 +420,35 @@ int compute_classes(smpq_ctx *ctx, const std::vector<int> &classes, double *q_re
         cudaMemcpyAsync(d_rhs_class, h_rhs.data(), 3 * (size_t)B * sizeof(int), cudaMemcpyHostToDevice, st);
         if (kind == 1) { // source D_W^dag b of the normal equations
             double2 *b = (double2 *)ctx->ws[W_SRC].p;
-            launch_class_source(ctx->V, B, BC, spec.d_colour, d_rhs_class, d_src_comp, b, st);
-            launch_dslash<double>(ctx->geom, ctx->U64.p, b, (void *)spec.d_src_field, B, BC, 1, ctx->opt.kappa, st);
+            launch_class_source(ctx->V, Bb, BC, spec.d_colour, d_rhs_class, d_src_comp, b, st);
+            launch_dslash<double>(ctx->geom, ctx->U64.p, b, (void *)spec.d_src_field, Bb, BC, 1, ctx->opt.kappa, st);
             ctx->launches += 2;
         }
-        if (project) lowmodes_source(ctx, (double2 *)ctx->ws[W_SRC].p, B, BC, d_rhs_class, d_src_comp, st);
+        if (project) lowmodes_source(ctx, (double2 *)ctx->ws[W_SRC].p, Bb, BC, d_rhs_class, d_src_comp, st);
         SolveOut out;
         rc = multishift_solve(ctx, spec, &out);
         if (rc) return rc;
         if (kind == 0) {
             if (project)
-                lowmodes_add_c0b(ctx, n_sup, B, BC, spec.d_supsite, d_rhs_class, (const double2 *)ctx->ws[W_SRC].p,
+                lowmodes_add_c0b(ctx, n_sup, Bb, BC, spec.d_supsite, d_rhs_class, (const double2 *)ctx->ws[W_SRC].p,
                                  out.y, st);
             else
-                launch_add_c0b(n_sup, B, BC, spec.d_supsite, d_rhs_class, d_src_comp, spec.d_colour, ctx->c0, out.y,
+                launch_add_c0b(n_sup, Bb, BC, spec.d_supsite, d_rhs_class, d_src_comp, spec.d_colour, ctx->c0, out.y,
                                st);
             if (full_sup) { // y is a whole-lattice field: z = D_W y everywhere, read at the members
-                if ((rc = ensure(ctx, ctx->ws[W_OUT], (size_t)ctx->V * 12 * B * sizeof(double2)))) return rc;
+                if ((rc = ensure(ctx, ctx->ws[W_OUT], (size_t)ctx->V * 12 * Bb * sizeof(double2)))) return rc;
                 double2 *z = (double2 *)ctx->ws[W_OUT].p;
-                launch_dslash<double>(ctx->geom, ctx->U64.p, out.y, z, B, BC, 0, ctx->opt.kappa, st);
-                launch_contract_full(z, ctx->V, B, BC, d_rhs_class, d_src_comp, (const int *)ctx->d_members.p,
+                launch_dslash<double>(ctx->geom, ctx->U64.p, out.y, z, Bb, BC, 0, ctx->opt.kappa, st);
+                launch_contract_full(z, ctx->V, Bb, BC, d_rhs_class, d_src_comp, (const int *)ctx->d_members.p,
                                      ctx->members, (double2 *)ctx->ws[W_QTERM].p, st);
                 ctx->launches += 1;
             } else {
-                launch_contract(ctx->geom, (const double *)ctx->U64.p, out.y, n_sup, B, BC, d_rhs_class,
+                launch_contract(ctx->geom, (const double *)ctx->U64.p, out.y, n_sup, Bb, BC, d_rhs_class,
                                 d_src_comp, (const int *)ctx->d_members.p, ctx->members, ctx->opt.kappa,
                                 (double2 *)ctx->ws[W_QTERM].p, st);
             }
         } else {
-            launch_trace_terms(out.y, n_sup, B, BC, d_rhs_class, d_src_comp, ctx->members,
+            launch_trace_terms(out.y, n_sup, Bb, BC, d_rhs_class, d_src_comp, ctx->members,
                                (double2 *)ctx->ws[W_QTERM].p, st);
         }
         ctx->launches += 2;
@@ -1127,11 +1134,13 @@ int smpq_time_dslash(smpq_ctx *ctx, int B, int dagger, int precision, int reps, 
     DeviceGuard dg(ctx->device);
     StreamEntry se(ctx, ctx->user_stream);
     cudaStream_t st = ctx->stream;
-    const size_t fb = dslash_field_bytes(ctx, precision, B);
-    if ((rc = ensure(ctx, ctx->ws[W_SRC], 2 * fb))) return rc;
+    // FP64: a block-fixed-point input (zeros) and a field of doubles
+    const bool fp64 = precision == SMPQ_FP64;
+    const size_t ob = dslash_field_bytes(ctx, precision, B), fb = fp64 ? (bf_field_bytes(ctx->V, B) + 255) / 256 * 256 : ob;
+    if ((rc = ensure(ctx, ctx->ws[W_SRC], fb + ob))) return rc;
     char *tin = (char *)ctx->ws[W_SRC].p, *tout = tin + fb;
-    cudaMemsetAsync(tin, 0x3F, 2 * fb, st);
-    // the FP64 / FP32 tile: the widest of 48, 12 and 1 that divides B
+    cudaMemsetAsync(tin, fp64 ? 0 : 0x3F, fb + ob, st);
+    // the FP32 tile: the widest of 48, 12 and 1 that divides B
     const int BC = B % 48 == 0 ? 48 : (B % 12 == 0 ? 12 : 1);
     const void *U = dslash_links(ctx, precision);
     // FP32 on tiles of 12 or more columns with staging 1: the neighbour sites staged in shared memory
@@ -1142,7 +1151,7 @@ int smpq_time_dslash(smpq_ctx *ctx, int B, int dagger, int precision, int reps, 
     }
     cudaError_t le = cudaSuccess;
     auto launch = [&]() {
-        if (precision == SMPQ_FP64) launch_dslash<double>(ctx->geom, U, tin, tout, B, BC, dagger, ctx->opt.kappa, st);
+        if (fp64) launch_dslash_bf(ctx->geom, ctx->Ubf.p, U, tin, (const double *)tin, (double *)tout, B, dagger, ctx->opt.kappa, st);
         else if (staged) {
             const cudaError_t e = launch_dslash_staged(ctx->geom, U, tin, tout, B, BC, dagger, ctx->opt.kappa,
                                                        (int *)ctx->d_err.p, st);

@@ -1,8 +1,8 @@
 // D_W in block fixed point: FP64 accuracy on the integer pipe.
 //
-// GB300 executes 2 FP64 operations per clock and SM, but 64 multiply-adds of
-// two 32-bit integers into a 64-bit sum (mad.wide: 2 cycles a warp against 66
-// for an FP64 FMA, measured).  The FP64 iterations therefore keep a site's 24
+// GB300 executes 2 FP64 operations per clock and SM: an FP64 FMA occupies an SM
+// quarter for 66 cycles a warp, a multiply-add of two 32-bit integers into a
+// 64-bit sum (mad.wide) for 4.5 (both measured).  The FP64 iterations therefore keep a site's 24
 // real numbers (12 complex components of one column) as 64-bit integers with
 // one exponent,
 //     value = v * 2^e,  |v| < 2^60, the largest at least 2^59,
@@ -19,9 +19,13 @@
 // high sum, in units of 2^64, is below sqrt(6) * 2^(61 + 60 - 64) and eight
 // hops below 2^61.3.
 //
-// Cycles a warp for one site and 32 columns: 8 hops of 228 mad.wide (2), 36
-// shifts and splits (4 and 3), 36 64-bit additions (2) and 21 loads come to
-// 5500; the 960 FP64 instructions that they replace take 63 000.
+// Bound by the integer pipe: 8 hops of 228 mad.wide and about 370 cycles of
+// shifts, splits, additions and loads come to 11 000 cycles a warp; the 960 FP64
+// instructions that they replace took 63 000.  Measured on 8^3x16 with 72 columns:
+// a solver launch of 300 us (1340 us in FP64); stand-alone with 12 columns 97 us
+// a call (261).  Not kept: products of the middle words in FP32 (1.6e-16 of the
+// result's norm instead of 1.2e-16), one copy of the hop for all directions (same
+// time), eight copies (15 % slower: instruction cache).
 #pragma once
 #include "wilson.cuh"
 
@@ -336,15 +340,93 @@ __device__ __forceinline__ void bf_wilson(const Geom &g, const int4 *__restrict_
     dir(std::integral_constant<int, 3>());
 }
 
+// the 9 exponents that a site's D_W reads: neighbours, exponents, the largest one
+struct BfStar {
+    int nb[8], en[8], eown, eref;
+    bool edge[8]; // the hop crosses an antiperiodic boundary
+    template <typename Off>
+    __device__ __forceinline__ BfStar(const Geom &g, const int *__restrict__ ein, const Off &off, int s) {
+        const SiteCoords xc(g, s);
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) {
+            const int n = g.n[mu], st = g.stride[mu], c = xc.x[mu];
+            const bool top = c == n - 1, bot = c == 0, anti = g.bcf[mu] < 0;
+            nb[2 * mu] = top ? s - (n - 1) * st : s + st;
+            nb[2 * mu + 1] = bot ? s + (n - 1) * st : s - st;
+            edge[2 * mu] = anti && top;
+            edge[2 * mu + 1] = anti && bot;
+        }
+        eown = eref = ein[off.exp(s)];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) en[k] = ein[off.exp(nb[k])];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) eref = max(eref, en[k]);
+    }
+};
+// acc += the two hops of direction MU
+template <int MU, bool DAG, typename Off>
+__device__ __forceinline__ void bf_dir(const BfStar &x, const int4 *__restrict__ U, const bfc *__restrict__ in,
+                                       const Off &off, int V, int s, int one, bfc acc[12]) {
+#pragma unroll 1
+    for (int bk = 0; bk < 2; ++bk) {
+        const bool back = bk != 0;
+        const int nb = back ? x.nb[2 * MU + 1] : x.nb[2 * MU], en = back ? x.en[2 * MU + 1] : x.en[2 * MU];
+        bf_hop<MU, DAG>(back, U, in, off, V, nb, back ? nb : s, min(x.eref - en, 63),
+                        back ? x.edge[2 * MU + 1] : x.edge[2 * MU], one, acc);
+    }
+}
+// The same by four groups of GT threads (thread t of each group: the same site
+// and column; every thread of the block calls it, `on` where there is a site),
+// for launches too small to hide one thread's eight hops: group q does
+// direction q, the sums go through shared memory (sm[4][6][GT]) and group q
+// keeps components 3 q .. 3 q + 2 in acc[0..2].  Integer sums: the bits are
+// those of bf_wilson.
+template <bool DAG, int GT, typename Off>
+__device__ __forceinline__ void bf_wilson_split(const Geom &g, const int4 *__restrict__ U, const bfc *__restrict__ in,
+                                                const int *__restrict__ ein, const Off &off, int s, bool on, int one,
+                                                bfc (*sm)[6][GT], bfc keep[3], int &eown, int &eref) {
+    const int q = threadIdx.x / GT, t = threadIdx.x % GT;
+    bfc acc[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) acc[c] = {0, 0};
+    eown = eref = BF_ZERO;
+    if (on) {
+        const BfStar x(g, ein, off, s);
+        eown = x.eown;
+        eref = x.eref;
+if (q == 0) bf_dir<0, DAG>(x, U, in, off, g.V, s, one, acc);
+        else if (q == 1) bf_dir<1, DAG>(x, U, in, off, g.V, s, one, acc);
+        else if (q == 2) bf_dir<2, DAG>(x, U, in, off, g.V, s, one, acc);
+        else bf_dir<3, DAG>(x, U, in, off, g.V, s, one, acc);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) { // upper half to groups 0 and 1, lower to 2 and 3
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 6; ++c) sm[q][c][t] = acc[6 * h + c];
+        __syncthreads();
+        if ((q >> 1) == h) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int k = 3 * (q & 1) + c;
+                bfc v = sm[0][k][t];
+#pragma unroll
+                for (int r = 1; r < 4; ++r) v = {v.x + sm[r][k][t].x, v.y + sm[r][k][t].y};
+                keep[c] = v;
+            }
+        }
+    }
+}
 // x = own - kappa acc in units of 2^eu, eu at least `least` (>= eown + 2, the
 // exponent of the block own); |x| < 2^60
-__device__ __forceinline__ void bf_dw(const bfc own[12], int eown, const bfc acc[12], int eref, const BfScal &k,
-                                      int least, int one, bfc x[12], int &eu) {
+template <int N>
+__device__ __forceinline__ void bf_dw(const bfc own[N], int eown, const bfc acc[N], int eref, const BfScal &k,
+                                      int least, int one, bfc x[N], int &eu) {
     const int eq = eref <= BF_ZERO / 2 ? BF_ZERO : eref + 4 + k.e + 64;
     eu = max(eq, least);
     const int n = eu - eown, m = eu - eq;
 #pragma unroll
-    for (int c = 0; c < 12; ++c) {
+    for (int c = 0; c < N; ++c) {
         long long qx = bf_mul(acc[c].x, k, one), qy = bf_mul(acc[c].y, k, one);
         if (m) { // (only for a tiny kappa)
             qx = bf_shr(qx, m);
@@ -355,6 +437,11 @@ __device__ __forceinline__ void bf_dw(const bfc own[12], int eown, const bfc acc
     if (eref >= BF_BAD / 2) eu = BF_BAD;
 }
 
+// sites times columns up to which a stand-alone D_W is split over four threads
+// each (one vector of 4^4: 48 against 58 us; 98 304 on 12 vectors of 8^3x16: 110
+// against 97 us, there the SMs are full.  A solve's launches gained nothing: D_ov
+// on 3 vectors of 8^3x16 13.6 against 13.2 ms)
+constexpr size_t BF_SPLIT_MAX = 40000;
 // thread -> (site, column) of the block-fixed-point kernels: blocks of about a
 // hundred threads, so that small lattices reach every SM (24 576 sites and
 // columns are 384 blocks); 128 registers a thread

@@ -285,8 +285,7 @@ static __device__ __noinline__ void dw_site_fp64(const Geom &g, const double2 *_
     }
 }
 
-// one thread per site and column in blocks of 32 (few columns: every warp on an
-// SM of its own) or 128 threads; bound by the integer pipe
+// one thread per site and column; bound by the integer pipe
 template <bool DAG>
 __global__ void __launch_bounds__(128, 4)
     dslash_bf_kernel(Geom g, const int4 *__restrict__ Ubf, const double2 *__restrict__ U64, const bfc *__restrict__ v,
@@ -306,10 +305,39 @@ __global__ void __launch_bounds__(128, 4)
     }
 #pragma unroll
     for (int c = 0; c < 12; ++c) own[c] = v[j + off(s, c)];
-    bf_dw(own, eown, acc, eref, ks, eown + 2, one, acc, eu);
+    bf_dw<12>(own, eown, acc, eref, ks, eown + 2, one, acc, eu);
 #pragma unroll
     for (int c = 0; c < 12; ++c)
         out[j + off(s, c)] = make_double2(bf_double(acc[c].x, eu), bf_double(acc[c].y, eu));
+}
+// four threads per site and column (bf_wilson_split), 32 of those per block: up to
+// BF_SPLIT_MAX of them, where one thread's eight hops in a row set the time
+template <bool DAG>
+__global__ void __launch_bounds__(128, 4)
+    dslash_bf_split_kernel(Geom g, const int4 *__restrict__ Ubf, const double2 *__restrict__ U64,
+                           const bfc *__restrict__ v, const int *__restrict__ e, const double2 *__restrict__ in,
+                           double2 *__restrict__ out, int B, BfScal ks, double kappa) {
+    __shared__ bfc sm[4][6][32];
+    const int q = threadIdx.x / 32;
+    const long i = blockIdx.x * 32l + threadIdx.x % 32;
+    const bool on = i < (long)g.V * B;
+    const int s = on ? (int)(i / B) : 0, j = on ? (int)(i % B) : 0;
+    const BfOff<0> off{g.V, B};
+    const int one = opaque_one();
+    bfc acc[3], own[3];
+    int eown, eref, eu;
+    bf_wilson_split<DAG, 32>(g, Ubf, v + j, e + j, off, s, on, one, sm, acc, eown, eref);
+    if (!on) return;
+    if (eref >= BF_BAD / 2) {
+        if (q == 0) dw_site_fp64(g, U64, in + j, out + j, s, B, DAG, kappa);
+        return;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) own[c] = v[j + off(s, 3 * q + c)];
+    bf_dw<3>(own, eown, acc, eref, ks, eown + 2, one, acc, eu);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        out[j + off(s, 3 * q + c)] = make_double2(bf_double(acc[c].x, eu), bf_double(acc[c].y, eu));
 }
 
 size_t bf_field_bytes(int V, int B) { return (size_t)V * B * (12 * sizeof(bfc) + sizeof(int)); }
@@ -322,17 +350,17 @@ void launch_abi_to_bf(const double *in, void *field, int V, int B, cudaStream_t 
 void launch_dslash_bf(const Geom &g, const void *Ubf, const void *U64, const void *field, const double *in,
                       double *out, int B, int dagger, double kappa, cudaStream_t st) {
     const long n = (long)g.V * B;
-    const int th = n < 152 * 128 * 4 ? 32 : 128;
-    const unsigned nb = (unsigned)((n + th - 1) / th);
+    const bool split = n <= (long)BF_SPLIT_MAX;
+    const unsigned nb = (unsigned)(split ? (n + 31) / 32 : (n + 127) / 128);
     const bfc *v = (const bfc *)field;
     const int *e = (const int *)(v + 12 * n);
     const BfScal ks = bf_scal(kappa);
-    if (dagger)
-        dslash_bf_kernel<true><<<nb, th, 0, st>>>(g, (const int4 *)Ubf, (const double2 *)U64, v, e,
-                                                  (const double2 *)in, (double2 *)out, B, ks, kappa);
-    else
-        dslash_bf_kernel<false><<<nb, th, 0, st>>>(g, (const int4 *)Ubf, (const double2 *)U64, v, e,
-                                                   (const double2 *)in, (double2 *)out, B, ks, kappa);
+    auto go = [&](auto kernel) {
+        kernel<<<nb, 128, 0, st>>>(g, (const int4 *)Ubf, (const double2 *)U64, v, e, (const double2 *)in,
+                                   (double2 *)out, B, ks, kappa);
+    };
+    if (split) dagger ? go(dslash_bf_split_kernel<true>) : go(dslash_bf_split_kernel<false>);
+    else dagger ? go(dslash_bf_kernel<true>) : go(dslash_bf_kernel<false>);
 }
 
 __global__ void __launch_bounds__(256) abi_to_float_kernel(const double2 *__restrict__ in, float2 *__restrict__ out,

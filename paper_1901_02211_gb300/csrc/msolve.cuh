@@ -97,10 +97,13 @@ struct Scal {
     int *act_rhs, *upd_rhs, *iters;                                  // [B]
     double *zeta, *zeta_prev;                                        // [n][B]
     int *act, *upd;                                                  // [n][B]
-    // per iteration of the history (row slot[j] of column j), [rows][n][B]: the
-    // shift's alpha_i, beta_i, zeta_{k+1} as its direction saw them (0, 1, 0
-    // in an iteration that left the direction alone)
-    double *ha, *hb, *hz;
+    // per iteration of the history (row slot[j] of column j): zeta_{k+1} and the
+    // zeta_k before it of every shift, [rows][n][B] (hz 0 in an iteration that
+    // left the shift's direction alone), alpha and beta of the column, [rows][B].
+    // The shift's own alpha_i = alpha zeta_{k+1} / zeta_k and beta_i = beta
+    // (zeta_{k+1} / zeta_k)^2 are formed from them at the end (their divisions
+    // were half of the scalar steps' FP64 work, which every launch waits for).
+    double *hz, *ho, *hal, *hbe;
     int *slot;    // [B] history row of the column's current iteration
     int slot_inc; // 1; 0 without a history (every row is row 0)
     int *flags; // [0] active rhs count, [1] residual replacement requested, [2] breakdown,
@@ -210,12 +213,12 @@ __device__ void s1_tile(int j0, double tt, double pp, const Scal &sc, const Shif
         for (int i = t / BC; i < sp.n; i += K) {
             const int ix = i * B + j;
             const size_t hx = row + (size_t)i * B;
-            if (!on || !sc.act[ix]) { sc.upd[ix] = 0; sc.ha[hx] = 0; continue; }
+            if (!on || !sc.act[ix]) { sc.upd[ix] = 0; continue; }
             double z = sc.zeta[ix], zp = sc.zeta_prev[ix];
             double den = a * bp * (zp - z) + zp * ap * (1.0 + sp.sig[i] * a);
             double zn = z * zp * ap / den;
             sc.hz[hx] = zn;
-            sc.ha[hx] = a * zn / z;
+            sc.ho[hx] = z;
             sc.upd[ix] = 1;
         }
     }
@@ -248,19 +251,16 @@ __device__ void s2_tile(int j0, double rrn, const Scal &sc, const ShiftParams &s
         const int q = t % BC, j = j0 + q;
         const size_t row = (size_t)sc.slot[j] * sp.n * B + j;
         const bool on = sc.upd_rhs[j];
-        const double r2 = sm[q], b = sm[BC + q], bb = sc.bb[j];
+        const double r2 = sm[q], bb = sc.bb[j];
         for (int i = t / BC; i < sp.n; i += K) {
             const int ix = i * B + j;
             const size_t hx = row + (size_t)i * B;
             if (!on || !sc.upd[ix]) {
                 if (on && sc.act[ix]) any[q] = 1;
-                sc.hb[hx] = 1;
                 sc.hz[hx] = 0;
                 continue;
             }
-            double z = sc.zeta[ix], zn = sc.hz[hx];
-            double w = zn / z;
-            sc.hb[hx] = b * w * w;
+            const double z = sc.ho[hx], zn = sc.hz[hx];
             sc.zeta_prev[ix] = z;
             sc.zeta[ix] = zn;
             int a = zn * zn * r2 > tol2 * bb;
@@ -271,6 +271,9 @@ __device__ void s2_tile(int j0, double rrn, const Scal &sc, const ShiftParams &s
     __syncthreads();
     if (t < BC) {
         const int j = j0 + t;
+        const size_t h = (size_t)sc.slot[j] * B + j;
+        sc.hal[h] = sc.alpha[j];
+        sc.hbe[h] = sm[BC + t];
         sc.slot[j] += sc.slot_inc;
         if (!sc.upd_rhs[j]) return;
         const double bb = sc.bb[j];
@@ -290,6 +293,8 @@ __device__ void s2_tile(int j0, double rrn, const Scal &sc, const ShiftParams &s
 // count == nullptr: no scalar step (the autotuner's timing launches).
 struct Fuse {
     int *count; // [tiles] blocks of the tile that have stored their partials; back to 0 after each launch
+    int *gcount; // [tiles][ngroups] the same for groups of 64 blocks
+    int ngroups;
     Scal sc;
     const ShiftParams *sp; // [lattices] each lattice's shifts (device memory)
     int B;                 // right-hand sides of the solve (stride of the shift-major scalars)
@@ -318,37 +323,88 @@ __device__ __forceinline__ bool last_block_of_tile(int *count, int G, bool wrote
 // Sum over the G blocks of an RHS tile (partial rows prow...) of each column, in
 // a fixed order (NT / BC lanes per column, then the lanes in order); every
 // thread of the block calls it, threads < BC receive their column's total.
-template <int BC, int NT> __device__ double tile_sum(const double *part, size_t prow, int G, double *sm) {
+// (rows: every step-th)
+template <int BC, int NT> __device__ double tile_sum(const double *part, size_t prow, int G, double *sm, int step = 1) {
     constexpr int K = NT / BC;
     const int t = threadIdx.x, jj = t % BC, k = t / BC;
     double v = 0;
     if (k < K)
-        for (int b = k; b < G; b += K) v += __ldcg(part + (prow + b) * BC + jj);
+        for (int b = k; b < G; b += K) v += __ldcg(part + (prow + (size_t)b * step) * BC + jj);
     if (k < K) sm[t] = v;
     __syncthreads();
     double tot = 0;
-    if (t < BC)
+    if constexpr (BC == 1) { // K = NT values: a tree (a chain of FP64 additions costs 70 cycles each)
+        for (int w = NT / 2; w > 0; w >>= 1) {
+            if (t < w) sm[t] += sm[t + w];
+            __syncthreads();
+        }
+        tot = sm[0];
+    } else if (t < BC) {
         for (int q = 0; q < K; ++q) tot += sm[q * BC + t];
+    }
     __syncthreads();
     return tot;
 }
 
+// A tile with many blocks sums its rows in two levels (GROUPS): the last block of
+// each 64 sums their rows into the first of them, the last of those sums the
+// groups.  In one level one SM adds G x BC numbers at 2 FP64 additions a clock:
+// for 16^3x32 (G = 6554, 48 columns) 80 us at the end of every launch.  The
+// float-float iterations keep one level, and with it the order of their sums: the
+// mixed solve's q(x) follows every rounding of alpha there by 1e-9 of its norm.
+constexpr int GROUP = 64;
+// true in every thread of the block that arrives last of all; nv sums v[q]
+template <int BC, int NT, int NV>
+__device__ __forceinline__ bool last_in_groups(const Fuse &f, double *const *v, size_t prow, int G, double *sm) {
+    const int grp = blockIdx.x / GROUP, first = grp * GROUP, n = min(GROUP, G - first);
+    __shared__ int last;
+    if (threadIdx.x < BC) __threadfence();
+    __syncthreads();
+    int *gc = f.gcount + (size_t)blockIdx.y * f.ngroups + grp;
+    if (threadIdx.x == 0) {
+        last = atomicAdd(gc, 1) == n - 1;
+        if (last) *gc = 0;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        const double s = tile_sum<BC, NT>(v[q], prow + first, n, sm);
+        if (threadIdx.x < BC) v[q][(prow + first) * BC + threadIdx.x] = s;
+    }
+    return last_block_of_tile(f.count, (G + GROUP - 1) / GROUP, threadIdx.x < BC);
+}
+
 // end of lattice kernel A: the tile's last block runs the first scalar step
 // (lattice l, its tile's partial rows from prow)
-template <int BC, int NT>
-__device__ __forceinline__ void fuse_step1(const Fuse &f, int l, const double *part_t, const double *part_p,
-                                           size_t prow, int G, double *sm) {
-    if (!f.count || !last_block_of_tile(f.count, G, threadIdx.x < BC)) return;
-    const double tt = tile_sum<BC, NT>(part_t, prow, G, sm);
-    const double pp = tile_sum<BC, NT>(part_p, prow, G, sm);
+template <int BC, int NT, bool GROUPS = false>
+__device__ __forceinline__ void fuse_step1(const Fuse &f, int l, double *part_t, double *part_p, size_t prow, int G,
+                                           double *sm) {
+    if (!f.count) return;
+    int step = 1;
+    if (GROUPS && G > 4 * GROUP) {
+        double *const v[2] = {part_t, part_p};
+        if (!last_in_groups<BC, NT, 2>(f, v, prow, G, sm)) return;
+        step = GROUP;
+        G = (G + GROUP - 1) / GROUP;
+    } else if (!last_block_of_tile(f.count, G, threadIdx.x < BC)) return;
+    const double tt = tile_sum<BC, NT>(part_t, prow, G, sm, step);
+    const double pp = tile_sum<BC, NT>(part_p, prow, G, sm, step);
     s1_tile<BC, NT>(blockIdx.y * BC, tt, pp, f.sc, f.sp[l], f.B, sm);
 }
 // end of lattice kernel B: the tile's last block runs the second scalar step
-template <int BC, int NT>
-__device__ __forceinline__ void fuse_step2(const Fuse &f, int l, const double *part_r, size_t prow, int G,
-                                           double *sm) {
-    if (!f.count || !last_block_of_tile(f.count, G, threadIdx.x < BC)) return;
-    const double rr = tile_sum<BC, NT>(part_r, prow, G, sm);
+template <int BC, int NT, bool GROUPS = false>
+__device__ __forceinline__ void fuse_step2(const Fuse &f, int l, double *part_r, size_t prow, int G, double *sm) {
+    if (!f.count) return;
+    int step = 1;
+    if (GROUPS && G > 4 * GROUP) {
+        double *const v[1] = {part_r};
+        if (!last_in_groups<BC, NT, 1>(f, v, prow, G, sm)) return;
+        step = GROUP;
+        G = (G + GROUP - 1) / GROUP;
+    } else if (!last_block_of_tile(f.count, G, threadIdx.x < BC)) return;
+    const double rr = tile_sum<BC, NT>(part_r, prow, G, sm, step);
     s2_tile<BC, NT>(blockIdx.y * BC, rr, f.sc, f.sp[l], f.B, f.tol2, f.delta2, f.theta2, sm);
 }
 
@@ -466,7 +522,7 @@ __global__ void __launch_bounds__(TileMap<BC, NR>::THREADS, MinBlocks<T>::value)
         part_t[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
         part_p[(prow + blockIdx.x) * BC + threadIdx.x] = s2;
     }
-    fuse_step1<BC, TM::THREADS>(f, l, part_t, part_p, prow, G, sm);
+    fuse_step1<BC, TM::THREADS, !std::is_same<T, df64>::value>(f, l, part_t, part_p, prow, G, sm);
 }
 
 // r -= alpha (D_W^dag t + s0 p); partial |r|^2 (NR columns per thread)
@@ -528,7 +584,7 @@ __global__ void __launch_bounds__(TileMap<BC, NR>::THREADS, MinBlocks<T>::value)
     }
     double s1 = block_total<BC, NR>(ar, sm);
     if (threadIdx.x < BC) part_r[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
-    fuse_step2<BC, TM::THREADS>(f, l, part_r, prow, G, sm);
+    fuse_step2<BC, TM::THREADS, !std::is_same<T, df64>::value>(f, l, part_r, prow, G, sm);
 }
 
 // ------------------------------------------------------------------ FP32 D_W pair, neighbours staged
@@ -583,7 +639,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS, 3)
         part_t[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
         part_p[(prow + blockIdx.x) * BC + threadIdx.x] = s2;
     }
-    fuse_step1<BC, TM::THREADS>(f, l, part_t, part_p, prow, G, sm);
+    fuse_step1<BC, TM::THREADS, true>(f, l, part_t, part_p, prow, G, sm);
 }
 
 template <int BC, bool M>
@@ -629,7 +685,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS, 3)
     }
     const double s1 = block_sum<BC>(ar, sm);
     if (threadIdx.x < BC) part_r[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
-    fuse_step2<BC, TM::THREADS>(f, l, part_r, prow, G, sm);
+    fuse_step2<BC, TM::THREADS, true>(f, l, part_r, prow, G, sm);
 }
 
 // The float-float pair (the first phase of SMPQ_MIXED) with staged neighbours
@@ -679,7 +735,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS, MinBlocks<df64>::value)
         part_t[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
         part_p[(prow + blockIdx.x) * BC + threadIdx.x] = s2;
     }
-    fuse_step1<BC, TM::THREADS>(f, l, part_t, part_p, prow, G, sm);
+    fuse_step1<BC, TM::THREADS, false>(f, l, part_t, part_p, prow, G, sm);
 }
 
 template <int BC, bool M>
@@ -726,7 +782,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS, MinBlocks<df64>::value)
     }
     const double s1 = block_sum<BC>(ar, sm);
     if (threadIdx.x < BC) part_r[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
-    fuse_step2<BC, TM::THREADS>(f, l, part_r, prow, G, sm);
+    fuse_step2<BC, TM::THREADS, false>(f, l, part_r, prow, G, sm);
 }
 
 template <int BC, bool M> cudaError_t staged_df_attrs() {
@@ -813,9 +869,9 @@ __device__ __forceinline__ void update_p_tiles(int bx, int tpb, int V, size_t ti
 
 // ------------------------------------------------------------------ FP64 iterations
 // SMPQ_FP64: p, t and r in block fixed point (bfp.cuh), one thread per site and
-// column.  Bound by the integer pipe: about 6400 (A) and 7000 (B) cycles a warp;
-// in FP64 arithmetic the pair took 46.7 + 48 ms for 3072 sources on 8^3x16, and
-// a small lattice's 24 blocks of 256 threads as long as a large one's.
+// column.  Bound by the integer pipe: 300 us a launch for 72 columns of 8^3x16
+// (1340 us in FP64 arithmetic); 24 576 sites and columns take 30 us (325 us in
+// blocks of 256 threads, 4 tiles each: 24 blocks on 152 SMs).
 template <int BC>
 __global__ void __launch_bounds__(BfMap<BC>::THREADS)
     k_init_bf(Geom g, Source src, BFF r, BFF p, double *part, int G) {
@@ -876,7 +932,7 @@ __global__ void __launch_bounds__(BfMap<BC>::THREADS, BfMap<BC>::BLOCKS)
 #pragma unroll
         for (int c = 0; c < 12; ++c) own[c] = p.v[base + off(s, c)];
         ap += bf_norm2(own, eown, one);
-        bf_dw(own, eown, acc, eref, kappa, eown + 2, one, acc, e);
+        bf_dw<12>(own, eown, acc, eref, kappa, eown + 2, one, acc, e);
         bf_normalise(acc, e);
         at += bf_norm2(acc, e, one);
 #pragma unroll
@@ -889,7 +945,7 @@ __global__ void __launch_bounds__(BfMap<BC>::THREADS, BfMap<BC>::BLOCKS)
         part_t[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
         part_p[(prow + blockIdx.x) * BC + threadIdx.x] = s2;
     }
-    fuse_step1<BC, TM::THREADS>(f, l, part_t, part_p, prow, G, sm);
+    fuse_step1<BC, TM::THREADS, true>(f, l, part_t, part_p, prow, G, sm);
 }
 
 // r -= alpha (D_W^dag t + s0 p); partial |r|^2
@@ -922,7 +978,7 @@ __global__ void __launch_bounds__(BfMap<BC>::THREADS, BfMap<BC>::BLOCKS)
         for (int c = 0; c < 12; ++c) own[c] = t.v[base + off(s, c)];
         // the unit of A p = D_W^dag t + s0 p: its last term takes part in the choice
         const int ep = p.e[ebase + off.exp(s)], ew = ep + s0.e + 64;
-        bf_dw(own, eown, acc, eref, kappa, max(eown + 3, ew + 1), one, acc, eu);
+        bf_dw<12>(own, eown, acc, eref, kappa, max(eown + 3, ew + 1), one, acc, eu);
         const int nw = eu - ew;
         // r - alpha A p
         int er = r.e[ebase + off.exp(s)];
@@ -945,7 +1001,7 @@ __global__ void __launch_bounds__(BfMap<BC>::THREADS, BfMap<BC>::BLOCKS)
     }
     const double s1 = block_sum<BC, TM::THREADS>(ar, sm);
     if (threadIdx.x < BC) part_r[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
-    fuse_step2<BC, TM::THREADS>(f, l, part_r, prow, G, sm);
+    fuse_step2<BC, TM::THREADS, true>(f, l, part_r, prow, G, sm);
 }
 
 // Launch YP of an FP64 iteration: r on the support into the history (as
@@ -1105,7 +1161,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS, 3)
         part_t[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
         part_p[(prow + blockIdx.x) * BC + threadIdx.x] = s2;
     }
-    fuse_step1<BC, TileMap<BC>::THREADS>(f, l, part_t, part_p, prow, G, sm);
+    fuse_step1<BC, TileMap<BC>::THREADS, true>(f, l, part_t, part_p, prow, G, sm);
 }
 
 // r -= alpha (D_W^dag t + s0 p); partial |r|^2
@@ -1153,7 +1209,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS, 3)
     }
     const double s1 = block_sum<BC>(ar, sm);
     if (threadIdx.x < BC) part_r[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
-    fuse_step2<BC, TileMap<BC>::THREADS>(f, l, part_r, prow, G, sm);
+    fuse_step2<BC, TileMap<BC>::THREADS, true>(f, l, part_r, prow, G, sm);
 }
 
 // p = r + beta p on the lattice tiles of tile group bx, p in the half format
@@ -1246,7 +1302,7 @@ __global__ void __launch_bounds__(TileMap<BC, 2>::THREADS, 2)
         part_t[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
         part_p[(prow + blockIdx.x) * BC + threadIdx.x] = s2;
     }
-    fuse_step1<BC, TM::THREADS>(f, l, part_t, part_p, prow, G, sm);
+    fuse_step1<BC, TM::THREADS, true>(f, l, part_t, part_p, prow, G, sm);
 }
 
 template <typename HT, int BC, bool M>
@@ -1298,7 +1354,7 @@ __global__ void __launch_bounds__(TileMap<BC, 2>::THREADS, 2)
     }
     const double s1 = block_total<BC, 2>(ar, sm);
     if (threadIdx.x < BC) part_r[(prow + blockIdx.x) * BC + threadIdx.x] = s1;
-    fuse_step2<BC, TM::THREADS>(f, l, part_r, prow, G, sm);
+    fuse_step2<BC, TM::THREADS, true>(f, l, part_r, prow, G, sm);
 }
 
 // ------------------------------------------------------------------ the residual history
@@ -1311,7 +1367,7 @@ __global__ void __launch_bounds__(TileMap<BC, 2>::THREADS, 2)
 // Before, launch YP read and wrote n shifted directions and y (32 n + 32 bytes
 // a value) with 6 n FP64 operations on them: with 14 shifts on 9/16 of the
 // lattice (r = 2) two thirds of a mixed solve (2.1 / 0.52 ms per FP64-accurate
-// / FP32 iteration of three lattices; the copy takes 0.3 / 0.13 ms).
+// / FP32 iteration of three lattices; the copy and p take 0.15 / 0.06 ms).
 //
 // FP64-accurate iterations (k_hist_w, k_hist_y, k_hist_p): over n iterations k
 // (r_k the residual after iteration k), with the scalars run backwards from
@@ -1365,8 +1421,21 @@ __device__ __forceinline__ double hi_lo(double v) {
     const float h = (float)v;
     return __hiloint2double(__float_as_int((float)(v - (double)h)), __float_as_int(h));
 }
+// alpha_i and beta_i of shift i in row k (0 and 1 where its direction was left alone)
+__device__ __forceinline__ void shift_scalars(const Scal &sc, int k, int i, int j, int nshift, int B, double &a,
+                                              double &b, double &z) {
+    const size_t o = ((size_t)k * nshift + i) * B + j;
+    z = sc.hz[o];
+    a = 0;
+    b = 1;
+    if (z != 0) {
+        const double zo = sc.ho[o], w = z / zo;
+        a = sc.hal[(size_t)k * B + j] * z / zo;
+        b = sc.hbe[(size_t)k * B + j] * w * w;
+    }
+}
 // The weights of a chunk of n iterations, one thread per shift and column of a
-// lattice (columns j0 <= j < j0 + Bl): hz <- c_i zeta_k S_{k+1}, ha <- zeta_k
+// lattice (columns j0 <= j < j0 + Bl): hz <- c_i zeta_k S_{k+1}, ho <- zeta_k
 // P_{k+1} (as two FP32 values); v0 <- c_i S_0, d0 <- P_0.
 __global__ void k_hist_w(int n, int nshift, int B, int j0, int Bl, const ShiftParams *__restrict__ sp, Scal sc,
                          double *__restrict__ v0, double *__restrict__ d0) {
@@ -1379,9 +1448,10 @@ __global__ void k_hist_w(int n, int nshift, int B, int j0, int Bl, const ShiftPa
     size_t o = (size_t)n * step + (size_t)i * B + j;
     for (int k = n - 1; k >= 0; --k) {
         o -= step;
-        const double a = sc.ha[o], b = sc.hb[o], z = sc.hz[o];
+        double a, b, z;
+        shift_scalars(sc, k, i, j, nshift, B, a, b, z);
         sc.hz[o] = c * (z * S);
-        sc.ha[o] = hi_lo(z * P);
+        sc.ho[o] = hi_lo(z * P);
         S = fma(b, S, a);
         P *= b;
     }
@@ -1467,7 +1537,7 @@ __global__ void __launch_bounds__(256) k_hist_y(HistLat L, const double *__restr
 // block at once, and serve the HROWS values of a thread from there (read from
 // global memory shift by shift they were the latency of the whole kernel: 100
 // ms of a 266 ms solve of three r = 2 lattices).
-constexpr int HROWS = 2, HK = 2, NG = 14;
+constexpr int HROWS = 2, NG = 14;
 template <int BC, typename V> struct HistTile {
     typedef TileMap<BC> TM;
     int jj, j, cls;      // column within the tile and the solve, its class
@@ -1485,6 +1555,7 @@ template <int BC, typename V> struct HistTile {
         }
     }
     // the scalars of iterations k0.. and shifts i0.. of the tile's columns (zeros beyond the last)
+    template <int HK>
     __device__ __forceinline__ static void load(const HistLat &L, const V *__restrict__ c, int k0, int i0,
                                                 V (*sm)[NG][BC], V zero) {
         for (int t = threadIdx.x; t < HK * NG * BC; t += TM::THREADS) {
@@ -1509,6 +1580,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_p(HistLat L, cons
                                                                  const double *__restrict__ d0,
                                                                  double2 *__restrict__ ps,
                                                                  float2 *__restrict__ ps32) {
+    constexpr int HK = 8;
     __shared__ double sm[HK][NG][BC];
     const HistTile<BC, double> T(L);
     for (int i0 = 0; i0 < L.nshift; i0 += NG) {
@@ -1534,7 +1606,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_p(HistLat L, cons
             }
             for (int k0 = 0; k0 < L.n; k0 += HK) {
                 __syncthreads();
-                HistTile<BC, double>::load(L, hp, k0, i0, sm, 0.0);
+                HistTile<BC, double>::template load<HK>(L, hp, k0, i0, sm, 0.0);
                 __syncthreads();
                 if (!T.ok[q]) continue;
 #pragma unroll
@@ -1577,12 +1649,14 @@ __global__ void k_hist_coef(int n, int nshift, int B, int j0, int Bl, const Shif
     const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (t >= (size_t)n * nshift * Bl) return;
     const size_t ki = t / Bl; // row * nshift + shift
-    const size_t o = ki * B + j0 + t % Bl;
-    const double ca = sp->c[ki % nshift] * sc.ha[o], w = hi_lo(ca);
-    sc.ha[o] = ca;
+    const int i = (int)(ki % nshift), j = j0 + (int)(t % Bl);
+    double a, b, z;
+    shift_scalars(sc, (int)(ki / nshift), i, j, nshift, B, a, b, z);
+    const size_t o = ki * B + j;
+    const double ca = sp->c[i] * a, w = hi_lo(ca);
+    sc.ho[o] = ca;
     // a converged shift's row (alpha 0) leaves y and its direction alone
-    ct[o] = make_float4(__int_as_float(__double2loint(w)), __int_as_float(__double2hiint(w)), (float)sc.hz[o],
-                        (float)sc.hb[o]);
+    ct[o] = make_float4(__int_as_float(__double2loint(w)), __int_as_float(__double2hiint(w)), (float)z, (float)b);
 }
 
 // A chunk of FP32 iterations: y += c_i alpha_i p_i, p_i = zeta r + beta p_i for
@@ -1597,6 +1671,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_run(HistLat L, co
                                                                    const float4 *__restrict__ ct,
                                                                    float2 *__restrict__ ps32,
                                                                    double2 *__restrict__ y, bool last) {
+    constexpr int HK = EXACT ? 2 : 4;
     __shared__ float4 sm[HK][NG][BC];
     __shared__ double sa[EXACT ? HK : 1][NG][BC];
     const HistTile<BC, float4> T(L);
@@ -1619,8 +1694,8 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_run(HistLat L, co
         }
         for (int k0 = 0; k0 < L.n; k0 += HK) {
             __syncthreads();
-            HistTile<BC, float4>::load(L, ct, k0, i0, sm, make_float4(0.f, 0.f, 0.f, 0.f));
-            if constexpr (EXACT) HistTile<BC, double>::load(L, ca, k0, i0, sa, 0.0);
+            HistTile<BC, float4>::template load<HK>(L, ct, k0, i0, sm, make_float4(0.f, 0.f, 0.f, 0.f));
+            if constexpr (EXACT) HistTile<BC, double>::template load<HK>(L, ca, k0, i0, sa, 0.0);
             __syncthreads();
             float2 rv[HK][HROWS];
 #pragma unroll
@@ -1946,7 +2021,9 @@ template <int BC> struct Solve {
     float4 *hct = nullptr;
     double tol2;
     int *hflags = nullptr;
-    int *count = nullptr;       // [nchunk] arrival counters of the fused scalar steps
+    int *count = nullptr;       // [nchunk] arrival counters of the fused scalar steps, [nchunk][ngroups] of groups
+    int ngroups = 1;
+    std::vector<int> rows1;     // per lattice: the most partial rows a launch has per tile
     double2 *x64 = nullptr;     // base-system solution in FP64 (true residual), nullable
     double *true_rr = nullptr;  // [B] |b - (A + s0) x64|^2
     int iters = 0, nrel = 0;
@@ -1999,7 +2076,8 @@ template <int BC> struct Solve {
             // partial rows per tile: the most blocks any launch has per tile (the
             // D_W launches at one tile per block have nt1; the support kernels Gs1)
             const int ntb = (V[l] + BfMap<BC>::SPB - 1) / BfMap<BC>::SPB;
-            npart += (size_t)nch[l] * std::max(std::max(nt1[l], ntb), Gs1[l]) * BC;
+            rows1.push_back(std::max(std::max(nt1[l], ntb), Gs1[l]));
+            npart += (size_t)nch[l] * rows1[l] * BC;
             sph[l] = in[l].sp;
         }
         tpb_hi = std::max(1, in[0].spec->tpb_hi > 0 ? in[0].spec->tpb_hi : TPB);
@@ -2013,17 +2091,20 @@ template <int BC> struct Solve {
         int rc;
         if ((rc = ensure(ctx, ws[W_PART], 3 * npart * sizeof(double)))) return rc;
         const size_t nscal = (size_t)B * 8 + (size_t)nshift * B * 2;
-        const size_t nint = (size_t)B * 4 + (size_t)nshift * B * 2 + 12 + (size_t)nchunk;
+        ngroups = 1;
+        for (int l = 0; l < nl; ++l) ngroups = std::max(ngroups, (rows1[l] + GROUP - 1) / GROUP);
+        const size_t nint = (size_t)B * 4 + (size_t)nshift * B * 2 + 12 + (size_t)nchunk * (1 + ngroups);
         if (shifts && (rc = plan_history())) return rc;
         const size_t rowlen = (size_t)nshift * B;
-        if ((rc = ensure(ctx, ws[W_HCOEF], (size_t)hrows * rowlen * (3 * sizeof(double) + sizeof(float4)) +
-                                                (((size_t)hrows + 1) * B + 2 * rowlen) * sizeof(double))))
+        if ((rc = ensure(ctx, ws[W_HCOEF], (size_t)hrows * rowlen * (2 * sizeof(double) + sizeof(float4)) +
+                                                ((3 * (size_t)hrows + 1) * B + 2 * rowlen) * sizeof(double))))
             return rc;
         hct = (float4 *)ws[W_HCOEF].p;
-        sc.ha = (double *)(hct + hrows * rowlen);
-        sc.hb = sc.ha + hrows * rowlen;
-        sc.hz = sc.hb + hrows * rowlen;
-        hw = sc.hz + hrows * rowlen;
+        sc.hz = (double *)(hct + hrows * rowlen);
+        sc.ho = sc.hz + hrows * rowlen;
+        sc.hal = sc.ho + hrows * rowlen;
+        sc.hbe = sc.hal + (size_t)hrows * B;
+        hw = sc.hbe + (size_t)hrows * B;
         hv0 = hw + ((size_t)hrows + 1) * B;
         hd0 = hv0 + rowlen;
         sc.slot_inc = shifts ? 1 : 0;
@@ -2067,7 +2148,7 @@ template <int BC> struct Solve {
             cudaGetLastError();
             return set_err(ctx, SMPQ_ENOMEM, "pinned host flags");
         }
-        cudaMemsetAsync(sc.flags, 0, (12 + (size_t)nchunk) * sizeof(int), st); // flags, counter, arrivals
+        cudaMemsetAsync(sc.flags, 0, (12 + (size_t)nchunk * (1 + ngroups)) * sizeof(int), st); // flags, counter, arrivals
         return SMPQ_OK;
     }
 
@@ -2263,9 +2344,9 @@ template <int BC> struct Solve {
             float2 *ps32 = (float2 *)ws[W_PS32].p + s0[l];
             const unsigned nb = (unsigned)((L.ne + 255) / 256);
             k_hist_y<C, BC><<<nb, 256, 0, st>>>(L, hw, hv0, ps, y + s0[l]);
-            if (next == 1) k_hist_p<C, BC, false><<<hist_grid<BC>(L), TileMap<BC>::THREADS, 0, st>>>(L, sc.ha, hd0, ps, ps32);
+            if (next == 1) k_hist_p<C, BC, false><<<hist_grid<BC>(L), TileMap<BC>::THREADS, 0, st>>>(L, sc.ho, hd0, ps, ps32);
             if constexpr (std::is_same<C, df64c>::value)
-                if (next == 2) k_hist_p<C, BC, true><<<hist_grid<BC>(L), TileMap<BC>::THREADS, 0, st>>>(L, sc.ha, hd0, ps, ps32);
+                if (next == 2) k_hist_p<C, BC, true><<<hist_grid<BC>(L), TileMap<BC>::THREADS, 0, st>>>(L, sc.ho, hd0, ps, ps32);
         }
         return hist_next(next == 0, 1 + (next ? 3 : 2) * nl);
     }
@@ -2283,8 +2364,8 @@ template <int BC> struct Solve {
             float2 *ps32 = (float2 *)ws[W_PS32].p + s0[l];
             const dim3 nb = hist_grid<BC>(L);
             const int TH = TileMap<BC>::THREADS;
-            if (exact) k_hist_run<BC, true><<<nb, TH, 0, st>>>(L, sc.ha, hct, ps32, y + s0[l], last);
-            else k_hist_run<BC, false><<<nb, TH, 0, st>>>(L, sc.ha, hct, ps32, y + s0[l], last);
+            if (exact) k_hist_run<BC, true><<<nb, TH, 0, st>>>(L, sc.ho, hct, ps32, y + s0[l], last);
+            else k_hist_run<BC, false><<<nb, TH, 0, st>>>(L, sc.ho, hct, ps32, y + s0[l], last);
         }
         return hist_next(last, 2 * nl);
     }
@@ -2382,8 +2463,8 @@ template <int BC> struct Solve {
             }
         }
         // the scalar steps ride on the last block of each RHS tile of launches A and B
-        const Fuse f1{count, sc, spd, B, 0.0, 0.0, 0.0};
-        const Fuse f2{count, sc, spd, B, tol2, delta2, theta2};
+        const Fuse f1{count, count + nchunk, ngroups, sc, spd, B, 0.0, 0.0, 0.0};
+        const Fuse f2{count, count + nchunk, ngroups, sc, spd, B, tol2, delta2, theta2};
         int gyp, tyy;
         const Lats Lyp = lats_yp(fixed_point ? BfMap<BC>::SPB : TileMap<BC>::SPB, &gyp, &tyy);
         C *hbase = shifts ? (C *)ctx->ws[W_HIST].p : nullptr;
