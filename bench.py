@@ -73,11 +73,11 @@ def _peaks():
 
 def _src_hash(kernel=""):
     """Hash of the files that define a solver kernel (wilson.cuh, df64.cuh,
-    device.cuh, msolve.cu, and stage.cuh for the staged FP32 kernels `*_st`):
+    device.cuh, msolve.cuh, and stage.cuh for the staged FP32 kernels `*_st`):
     traffic figures taken on other sources are void."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1901_02211_gb300", "csrc")
-    files = ["df64.cuh", "device.cuh", "msolve.cu", "wilson.cuh"] + (["stage.cuh"] if "_st[" in kernel else [])
+    files = ["df64.cuh", "device.cuh", "msolve.cuh", "wilson.cuh"] + (["stage.cuh"] if "_st[" in kernel else [])
     for f in files:
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
@@ -262,7 +262,7 @@ def _alu_peaks(dev):
 def _kernel_table(prec, stats, V, B, peak_hbm, peak_kind, alu):
     """Per solver kernel: average CUDA-event time per launch (profiled step),
     algorithmic bytes per launch (spinor fields read and written + links, as in
-    the module docstring of msolve.cu) against the measured HBM bandwidth, and
+    the module docstring of msolve.cuh) against the measured HBM bandwidth, and
     for the FP64-accurate kernels their arithmetic against the measured ALU peak."""
     from paper_1901_02211_gb300 import smpq
     link32, link64 = 4 * 9 * 8, 4 * 9 * 16

@@ -147,7 +147,7 @@ void set_geom(smpq_ctx *ctx) {
 struct Shape {
     int bc, tpb_hi, tpb_lo, nr, staged;
 };
-constexpr int TPB_DEFAULT = 4;    // tiles per block of the FP32 / half / FP64 D_W launches (msolve.cu)
+constexpr int TPB_DEFAULT = 4;    // tiles per block of the FP32 / half / FP64 D_W launches (msolve.cuh)
 constexpr int TPB_DEFAULT_HI = 2; // of the float-float ones (the tuner's usual choice on a GB300)
 
 std::string device_key(int dev) {

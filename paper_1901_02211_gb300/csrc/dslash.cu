@@ -119,9 +119,7 @@ template <typename T> void launch_from_tiled(const void *in, double *out, int V,
                                                                        (double2 *)out, V, B, BC);
 }
 template void launch_to_tiled<double>(const double *, void *, int, int, int, cudaStream_t);
-template void launch_to_tiled<float>(const double *, void *, int, int, int, cudaStream_t);
 template void launch_from_tiled<double>(const void *, double *, int, int, int, cudaStream_t);
-template void launch_from_tiled<float>(const void *, double *, int, int, int, cudaStream_t);
 
 // ------------------------------------------------------------------ stand-alone dslash
 template <typename T, bool DAG, int BC>

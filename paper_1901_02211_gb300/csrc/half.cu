@@ -8,7 +8,7 @@
 //     first two, recomputed in FP32 at every use;
 //   - arithmetic and accumulation in FP32.
 // This file holds the stand-alone D_W of smpq_dslash and smpq_time_dslash; the
-// solver's half-storage iterations (msolve.cu) share the device code in
+// solver's half-storage iterations (msolve.cuh) share the device code in
 // half.cuh.
 //
 // Layouts (RHS tiles of BC columns, as the FP32 and FP64 fields):

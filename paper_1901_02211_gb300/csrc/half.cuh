@@ -1,5 +1,5 @@
 // Half-precision storage formats shared by the stand-alone D_W (half.cu) and
-// the solver's half-storage iterations (msolve.cu): FP16 or BF16 complex
+// the solver's half-storage iterations (msolve.cuh): FP16 or BF16 complex
 // components scaled by one FP32 norm per site and right-hand side, links as
 // rows 0 and 1 (reconstruct-12), FP32 arithmetic.  Layout of a field of B
 // columns in RHS tiles of BC: components [j / BC][V][12][BC] (one complex

@@ -145,7 +145,7 @@ cudaError_t launch_dslash_staged(const Geom &g, const void *U, const void *in, v
 void launch_dslash_half(int prec, const Geom &g, const void *U, const void *in, void *out, int B, int dagger,
                         double kappa, cudaStream_t st);
 
-// msolve.cu : multi-shift CG over a batch (see msolve.cu for the contract)
+// msolve.cuh : multi-shift CG over a batch (see msolve.cuh for the contract)
 struct SolveSpec {
     int B, BC;                 // right-hand sides and tile width
     int prec;                  // SMPQ_FP64 / SMPQ_FP32 / SMPQ_MIXED
