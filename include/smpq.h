@@ -242,7 +242,9 @@ int smpq_build_sources(smpq_ctx *ctx, int r, int mode, int *n_classes);
 int smpq_colour_sites(const int dims[4], int r, int mode, int *colour, int *n_classes);
 
 /* D_W (or gamma_5 D_W gamma_5 = D_W^dag if dagger) applied to B fields
- * (Sec. 2.1, Eq. 3), computed in `precision`: SMPQ_FP64 or SMPQ_FP32 kernels,
+ * (Sec. 2.1, Eq. 3), computed in `precision`: SMPQ_FP64 (in 64-bit integers with
+ * one exponent per site and rhs, or in FP64 arithmetic where a component is too
+ * small for that: every component as accurate as FP64 arithmetic gives it), SMPQ_FP32,
  * or SMPQ_FP16N / SMPQ_BF16N (the input is rounded to the half format on the
  * device, the result leaves the kernel in that format and is widened back to
  * FP64).  in/out FP64 at the ABI: double[V][4][3][B][2], host or device
@@ -254,8 +256,8 @@ int smpq_dslash(smpq_ctx *ctx, const double *in, double *out, int B, int dagger,
  * (SMPQ_FP64: block fixed point, 64-bit integers with one exponent per site and
  * rhs, written as doubles; SMPQ_FP32, SMPQ_FP16N or SMPQ_BF16N), in the RHS tile
  * the library picks for B.  The input and output fields are scratch in the
- * context's workspace, set once to the byte 0x3F (SMPQ_FP64: 0; finite values in
- * every format; the values do not change the work).  Two untimed launches, then
+ * context's workspace, set once to the byte 0x3F (SMPQ_FP64: to the blocks of
+ * such doubles; finite values in every format, which do not change the work).  Two untimed launches, then
  * `reps` (>= 1) launches back to back on the context's stream between two
  * CUDA events.  *ms (nullable): average milliseconds per launch; *bytes
  * (nullable): algorithmic bytes of one launch, V * B * (spinor bytes read +

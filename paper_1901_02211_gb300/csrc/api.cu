@@ -1092,7 +1092,8 @@ int smpq_dslash(smpq_ctx *ctx, const double *in, double *out, int B, int dagger,
     const size_t n = (size_t)ctx->V * 12 * B;
     const size_t fb = dslash_field_bytes(ctx, precision, B);
     // host buffers: staged copies of in and out; device: the caller's
-    const size_t bfb = precision == SMPQ_FP64 ? bf_field_bytes(ctx->V, B) : 0;
+    const bool bf = precision == SMPQ_FP64 && bf_dslash(ctx->opt.kappa);
+    const size_t bfb = bf ? bf_field_bytes(ctx->V, B) : 0;
     const bool apart = !on_device || in + 2 * n <= out || out + 2 * n <= in;
     const size_t stage = on_device ? 0 : n * 16;
     if ((rc = ensure(ctx, ctx->ws[W_SRC], 2 * stage + std::max(2 * fb, bfb)))) return rc;
@@ -1105,10 +1106,10 @@ int smpq_dslash(smpq_ctx *ctx, const double *in, double *out, int B, int dagger,
     }
     const void *U = dslash_links(ctx, precision);
     double *dout = on_device ? out : abi;
-    if (precision == SMPQ_FP64 && apart) {
+    if (bf && apart) {
         launch_abi_to_bf(din, tin, ctx->V, B, st);
         launch_dslash_bf(ctx->geom, ctx->Ubf.p, U, tin, din, dout, B, dagger, ctx->opt.kappa, st);
-    } else if (precision == SMPQ_FP64) { // overlapping fields: through copies of both
+    } else if (precision == SMPQ_FP64) { // small kappa or overlapping fields: through copies of both
         launch_to_tiled<double>(din, tin, ctx->V, B, 1, st);
         launch_dslash<double>(ctx->geom, U, tin, tout, B, 1, dagger, ctx->opt.kappa, st);
         launch_from_tiled<double>(tout, dout, ctx->V, B, 1, st);
@@ -1134,14 +1135,16 @@ int smpq_time_dslash(smpq_ctx *ctx, int B, int dagger, int precision, int reps, 
     DeviceGuard dg(ctx->device);
     StreamEntry se(ctx, ctx->user_stream);
     cudaStream_t st = ctx->stream;
-    // FP64: a block-fixed-point input (zeros) and a field of doubles
-    const bool fp64 = precision == SMPQ_FP64;
-    const size_t ob = dslash_field_bytes(ctx, precision, B), fb = fp64 ? (bf_field_bytes(ctx->V, B) + 255) / 256 * 256 : ob;
+    const bool fp64 = precision == SMPQ_FP64, bf = fp64 && bf_dslash(ctx->opt.kappa);
+    const size_t ob = dslash_field_bytes(ctx, precision, B), fb = bf ? (bf_field_bytes(ctx->V, B) + 255) / 256 * 256 : ob;
     if ((rc = ensure(ctx, ctx->ws[W_SRC], fb + ob))) return rc;
     char *tin = (char *)ctx->ws[W_SRC].p, *tout = tin + fb;
-    cudaMemsetAsync(tin, fp64 ? 0 : 0x3F, fb + ob, st);
+    cudaMemsetAsync(tin, 0x3F, fb + ob, st);
+    // block fixed point: the input is such doubles, converted (all components of
+    // one size: no site needs the FP64 arithmetic, which alone would read `in`)
+    if (bf) launch_abi_to_bf((const double *)tout, tin, ctx->V, B, st);
     // the FP32 tile: the widest of 48, 12 and 1 that divides B
-    const int BC = B % 48 == 0 ? 48 : (B % 12 == 0 ? 12 : 1);
+    const int BC = fp64 ? 1 : B % 48 == 0 ? 48 : (B % 12 == 0 ? 12 : 1);
     const void *U = dslash_links(ctx, precision);
     // FP32 on tiles of 12 or more columns with staging 1: the neighbour sites staged in shared memory
     const bool staged = precision == SMPQ_FP32 && BC >= 12 && ctx->opt.staging == 1;
@@ -1151,7 +1154,8 @@ int smpq_time_dslash(smpq_ctx *ctx, int B, int dagger, int precision, int reps, 
     }
     cudaError_t le = cudaSuccess;
     auto launch = [&]() {
-        if (fp64) launch_dslash_bf(ctx->geom, ctx->Ubf.p, U, tin, (const double *)tin, (double *)tout, B, dagger, ctx->opt.kappa, st);
+        if (bf) launch_dslash_bf(ctx->geom, ctx->Ubf.p, U, tin, (const double *)tin, (double *)tout, B, dagger, ctx->opt.kappa, st);
+        else if (fp64) launch_dslash<double>(ctx->geom, U, tin, tout, B, BC, dagger, ctx->opt.kappa, st);
         else if (staged) {
             const cudaError_t e = launch_dslash_staged(ctx->geom, U, tin, tout, B, BC, dagger, ctx->opt.kappa,
                                                        (int *)ctx->d_err.p, st);

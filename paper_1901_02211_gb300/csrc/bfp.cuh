@@ -12,7 +12,11 @@
 // low word, is three mad.wide into 64-bit sums (high; middle twice); low times
 // low, about 2^-57 of the largest, is left out.  Sums are exact, so the hop's
 // error is that of its truncations, about 2^-56 of the largest component of
-// the nine sites, against 2^-53 of every partial sum in FP64.
+// the nine sites, against 2^-53 of every partial sum in FP64.  Relative to the
+// largest: a component that is smaller by 2^k and does not mix with it (unit or
+// diagonal links) has k bits less.  The solver's norms, residuals and tolerances
+// are those of whole vectors; the stand-alone D_W looks at every component
+// (bf_dw_fine).
 //   Bounds: a projected component is below 2^61, so its words are below 2^29
 // and 2^31, a link's 2^28 and 2^31.  Six products in a middle sum stay below
 // 6 * 2^60 + sqrt(6) * 2^59 < 2^63; the rows of a link have norm 1, so a hop's
@@ -22,7 +26,7 @@
 // Bound by the integer pipe: 8 hops of 228 mad.wide and about 370 cycles of
 // shifts, splits, additions and loads come to 11 000 cycles a warp; the 960 FP64
 // instructions that they replace took 63 000.  Measured on 8^3x16 with 72 columns:
-// a solver launch of 300 us (1340 us in FP64); stand-alone with 12 columns 97 us
+// a solver launch of 300 us (1340 us in FP64); stand-alone with 12 columns 100 us
 // a call (261).  Not kept: products of the middle words in FP32 (1.6e-16 of the
 // result's norm instead of 1.2e-16), one copy of the hop for all directions (same
 // time), eight copies (15 % slower: instruction cache).
@@ -120,9 +124,9 @@ __device__ __forceinline__ double bf_double(long long v, int e) {
     return __hiloint2double(hi + (e << 20), __double2loint(d));
 }
 
-// 24 doubles as a block (e = BF_BAD if some are not finite); wide: the nonzero
-// ones span more than 2^40
-__device__ __forceinline__ void bf_from_double(const double2 d[12], bfc v[12], int &e, bool &wide) {
+// 24 doubles as a block (e = BF_BAD if some are not finite); the result is the
+// span of the nonzero ones, as a difference of exponents
+__device__ __forceinline__ int bf_from_double(const double2 d[12], bfc v[12], int &e) {
     int top = 0, low = 0x7ff;
     bool any = false;
 #pragma unroll
@@ -138,7 +142,6 @@ __device__ __forceinline__ void bf_from_double(const double2 d[12], bfc v[12], i
             top = max(top, eb);
         }
     }
-    wide = any && top - low > 40;
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
         const double q[2] = {d[c].x, d[c].y};
@@ -154,6 +157,7 @@ __device__ __forceinline__ void bf_from_double(const double2 d[12], bfc v[12], i
         v[c] = bfc{r[0], r[1]};
     }
     e = top == 0x7ff ? BF_BAD : any ? top - 1082 : BF_ZERO;
+    return any ? top - low : 0;
 }
 
 // Brings a block with |v| < 2^60 and exponent e to the normal form.
@@ -224,6 +228,17 @@ template <int MU, int G> __device__ __forceinline__ void bf_lower(bfc w0, bfc w1
     l1 = {l1.x + G * b.x, l1.y + G * b.y};
 }
 
+// |re| and |im| of w in units of 2^48, in the low and the high half of a word
+// (one less for a negative number: bounds from below, so that a sum of eight
+// terms below 2^59 stays within 16 bits)
+__device__ __forceinline__ unsigned bf_size(bfc w) {
+    unsigned q, m;
+    asm("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(q) : "r"((int)(w.x >> 32)), "r"((int)(w.y >> 32)));
+    asm("prmt.b32 %0, %1, 0, 0xbb99;" : "=r"(m) : "r"(q)); // the signs, spread over each half
+    return q ^ m;
+}
+__device__ __forceinline__ unsigned bf_swap(unsigned z) { return (z >> 16) | (z << 16); }
+
 // acc += (1 + G g_mu) U psi(nb) (back = false, G = DAG ? 1 : -1) or (1 - G g_mu)
 // U^dag psi(nb) (back = true; as the conjugate of U^T conj(h)), its sign flipped
 // if flip; psi's block is shifted right by n bits to the common exponent, acc in
@@ -231,10 +246,12 @@ template <int MU, int G> __device__ __forceinline__ void bf_lower(bfc w0, bfc w1
 // code for each direction fits the instruction cache, eight do not (measured:
 // 210 against 178 ms for six classes of 8^3x16, "no instruction" the first stall).
 // links: int4 {re high, re low, im high, im low} per element
-template <int MU, bool DAG, typename Off>
+// SIZES: size[c] += the leading bits of |re| (low half) and |im| (high half) of
+// component c's term, in units of 2^48 (bf_small)
+template <int MU, bool DAG, bool SIZES = false, typename Off>
 __device__ __forceinline__ void bf_hop(bool back, const int4 *__restrict__ U, const bfc *__restrict__ in,
                                           const Off &off, int Vl, int nb, int ls, int n, bool flip, int one,
-                                          bfc acc[12]) {
+                                          bfc acc[12], unsigned *size = nullptr) {
     constexpr int GF = DAG ? 1 : -1;
     int hh[2][3][2], hl[2][3][2];
 #pragma unroll
@@ -286,6 +303,15 @@ __device__ __forceinline__ void bf_hop(bool back, const int4 *__restrict__ U, co
 #pragma unroll
         for (int s = 0; s < 2; ++s)
             w[s] = {madw((int)(rm[s] >> 32), one, rh[s]), madw((int)(im[s] >> 32), one, ih[s])};
+        if constexpr (SIZES) {
+            const unsigned z0 = bf_size(w[0]), z1 = bf_size(w[1]);
+            size[a] += z0;
+            size[3 + a] += z1;
+            // the lower half's terms (bf_lower): i w has re and im in turn
+            const unsigned l0 = MU == 0 || MU == 1 ? z1 : z0, l1 = MU == 0 || MU == 1 ? z0 : z1;
+            size[6 + a] += MU == 0 || MU == 2 ? bf_swap(l0) : l0;
+            size[9 + a] += MU == 0 || MU == 2 ? bf_swap(l1) : l1;
+        }
         if (back) {
             acc[a] = {acc[a].x + w[0].x, acc[a].y - w[0].y};
             acc[3 + a] = {acc[3 + a].x + w[1].x, acc[3 + a].y - w[1].y};
@@ -340,82 +366,164 @@ __device__ __forceinline__ void bf_wilson(const Geom &g, const int4 *__restrict_
     dir(std::integral_constant<int, 3>());
 }
 
-// the 9 exponents that a site's D_W reads: neighbours, exponents, the largest one
+// The stand-alone D_W's exponents carry in their lowest bit whether the nonzero
+// components of the site span 2^12 and more.
+__device__ __forceinline__ int bf_tag(int e, bool wide) { return 2 * e + wide; }
+// What it knows of a site before it reads any component: where it lies at the
+// lattice's edges, its exponent and the star's largest, whether every neighbour is
+// zero (D_W then changes nothing).  Neighbours and their exponents are formed again
+// in each hop: kept over the eight hops they were 160 bytes of spills.
 struct BfStar {
-    int nb[8], en[8], eown, eref;
-    bool edge[8]; // the hop crosses an antiperiodic boundary
+    unsigned edges; // bit 2 mu: last coordinate, bit 2 mu + 1: first one
+    int eown, eref;
+    bool alone;
+    bool uneven; // bf_dw_fine is likely to find a small component: tagged, or only one or two large neighbours
     template <typename Off>
-    __device__ __forceinline__ BfStar(const Geom &g, const int *__restrict__ ein, const Off &off, int s) {
+    __device__ __forceinline__ BfStar(const Geom &g, const int *__restrict__ tag, const Off &off, int s) {
         const SiteCoords xc(g, s);
+        edges = 0;
 #pragma unroll
-        for (int mu = 0; mu < 4; ++mu) {
-            const int n = g.n[mu], st = g.stride[mu], c = xc.x[mu];
-            const bool top = c == n - 1, bot = c == 0, anti = g.bcf[mu] < 0;
-            nb[2 * mu] = top ? s - (n - 1) * st : s + st;
-            nb[2 * mu + 1] = bot ? s + (n - 1) * st : s - st;
-            edge[2 * mu] = anti && top;
-            edge[2 * mu + 1] = anti && bot;
+        for (int mu = 0; mu < 4; ++mu)
+            edges |= (xc.x[mu] == g.n[mu] - 1 ? 1u : 0u) << (2 * mu) | (xc.x[mu] == 0 ? 2u : 0u) << (2 * mu);
+        int en[8], top = BF_ZERO, large = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            en[k] = tag[off.exp(neighbour(g, s, k))] >> 1;
+            top = max(top, en[k]);
         }
-        eown = eref = ein[off.exp(s)];
+        const int own = tag[off.exp(s)];
+        eown = own >> 1;
+        eref = max(eown, top);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) en[k] = ein[off.exp(nb[k])];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) eref = max(eref, en[k]);
+        for (int k = 0; k < 8; ++k) large += en[k] >= eref - 4;
+        alone = top <= BF_ZERO / 2;
+        uneven = !alone && ((own & 1) || large <= 2);
     }
+    // k = 2 mu: forward in direction mu, 2 mu + 1: backward
+    __device__ __forceinline__ int neighbour(const Geom &g, int s, int k) const {
+        const int st = g.stride[k >> 1], far = (g.n[k >> 1] - 1) * st;
+        const bool edge = edges >> k & 1;
+        return k & 1 ? (edge ? s + far : s - st) : (edge ? s - far : s + st);
+    }
+    // a block in the star is marked bad
+    __device__ __forceinline__ bool bad() const { return eref >= BF_BAD / 2; }
 };
-// acc += the two hops of direction MU
+// acc += the two hops of direction MU, size likewise (bf_hop)
 template <int MU, bool DAG, typename Off>
-__device__ __forceinline__ void bf_dir(const BfStar &x, const int4 *__restrict__ U, const bfc *__restrict__ in,
-                                       const Off &off, int V, int s, int one, bfc acc[12]) {
+__device__ __forceinline__ void bf_dir(const BfStar &x, const Geom &g, const int4 *__restrict__ U,
+                                       const bfc *__restrict__ in, const int *__restrict__ tag, const Off &off, int s,
+                                       int one, bfc acc[12], unsigned size[12]) {
+    const bool anti = g.bcf[MU] < 0;
 #pragma unroll 1
     for (int bk = 0; bk < 2; ++bk) {
-        const bool back = bk != 0;
-        const int nb = back ? x.nb[2 * MU + 1] : x.nb[2 * MU], en = back ? x.en[2 * MU + 1] : x.en[2 * MU];
-        bf_hop<MU, DAG>(back, U, in, off, V, nb, back ? nb : s, min(x.eref - en, 63),
-                        back ? x.edge[2 * MU + 1] : x.edge[2 * MU], one, acc);
+        const int k = 2 * MU + bk, nb = x.neighbour(g, s, k);
+        bf_hop<MU, DAG, true>(bk != 0, U, in, off, g.V, nb, bk ? nb : s, min(x.eref - (tag[off.exp(nb)] >> 1), 63),
+                              anti && (x.edges >> k & 1), one, acc, size);
     }
 }
-// The same by four groups of GT threads (thread t of each group: the same site
-// and column; every thread of the block calls it, `on` where there is a site),
-// for launches too small to hide one thread's eight hops: group q does
-// direction q, the sums go through shared memory (sm[4][6][GT]) and group q
-// keeps components 3 q .. 3 q + 2 in acc[0..2].  Integer sums: the bits are
-// those of bf_wilson.
+// The eight hops of the star x and their sizes, or (split) by four groups of GT
+// threads (thread t of each group: the same site and column; every thread of the
+// block calls it, `on` where there is something to do), for launches too small to
+// hide one thread's eight hops: group q does direction q, the sums go through
+// shared memory and group q keeps components 3 q .. 3 q + 2 in acc[0..2] and
+// size[0..2].  Integer sums: the bits are the same.
+template <bool DAG, typename Off>
+__device__ __forceinline__ void bf_hops(const BfStar &x, const Geom &g, const int4 *__restrict__ U,
+                                        const bfc *__restrict__ in, const int *__restrict__ tag, const Off &off, int s,
+                                        int one, bfc acc[12], unsigned size[12]) {
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        acc[c] = {0, 0};
+        size[c] = 0;
+    }
+    bf_dir<0, DAG>(x, g, U, in, tag, off, s, one, acc, size);
+    bf_dir<1, DAG>(x, g, U, in, tag, off, s, one, acc, size);
+    bf_dir<2, DAG>(x, g, U, in, tag, off, s, one, acc, size);
+    bf_dir<3, DAG>(x, g, U, in, tag, off, s, one, acc, size);
+}
+template <int GT> struct BfSplit { // in shared memory
+    bfc v[4][6][GT];
+    unsigned z[4][6][GT];
+};
 template <bool DAG, int GT, typename Off>
-__device__ __forceinline__ void bf_wilson_split(const Geom &g, const int4 *__restrict__ U, const bfc *__restrict__ in,
-                                                const int *__restrict__ ein, const Off &off, int s, bool on, int one,
-                                                bfc (*sm)[6][GT], bfc keep[3], int &eown, int &eref) {
+__device__ __forceinline__ void bf_hops_split(const BfStar &x, const Geom &g, const int4 *__restrict__ U,
+                                              const bfc *__restrict__ in, const int *__restrict__ tag,
+                                              const Off &off, int s, bool on, int one, BfSplit<GT> &sm,
+                                              bfc keep[3], unsigned zkeep[3]) {
     const int q = threadIdx.x / GT, t = threadIdx.x % GT;
     bfc acc[12];
+    unsigned size[12];
 #pragma unroll
-    for (int c = 0; c < 12; ++c) acc[c] = {0, 0};
-    eown = eref = BF_ZERO;
+    for (int c = 0; c < 12; ++c) {
+        acc[c] = {0, 0};
+        size[c] = 0;
+    }
     if (on) {
-        const BfStar x(g, ein, off, s);
-        eown = x.eown;
-        eref = x.eref;
-if (q == 0) bf_dir<0, DAG>(x, U, in, off, g.V, s, one, acc);
-        else if (q == 1) bf_dir<1, DAG>(x, U, in, off, g.V, s, one, acc);
-        else if (q == 2) bf_dir<2, DAG>(x, U, in, off, g.V, s, one, acc);
-        else bf_dir<3, DAG>(x, U, in, off, g.V, s, one, acc);
+        if (q == 0) bf_dir<0, DAG>(x, g, U, in, tag, off, s, one, acc, size);
+        else if (q == 1) bf_dir<1, DAG>(x, g, U, in, tag, off, s, one, acc, size);
+        else if (q == 2) bf_dir<2, DAG>(x, g, U, in, tag, off, s, one, acc, size);
+        else bf_dir<3, DAG>(x, g, U, in, tag, off, s, one, acc, size);
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) { // upper half to groups 0 and 1, lower to 2 and 3
         __syncthreads();
 #pragma unroll
-        for (int c = 0; c < 6; ++c) sm[q][c][t] = acc[6 * h + c];
+        for (int c = 0; c < 6; ++c) {
+            sm.v[q][c][t] = acc[6 * h + c];
+            sm.z[q][c][t] = size[6 * h + c];
+        }
         __syncthreads();
         if ((q >> 1) == h) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const int k = 3 * (q & 1) + c;
-                bfc v = sm[0][k][t];
+                bfc v = sm.v[0][k][t];
+                unsigned z = sm.z[0][k][t];
 #pragma unroll
-                for (int r = 1; r < 4; ++r) v = {v.x + sm[r][k][t].x, v.y + sm[r][k][t].y};
+                for (int r = 1; r < 4; ++r) {
+                    v = {v.x + sm.v[r][k][t].x, v.y + sm.v[r][k][t].y};
+                    z += sm.z[r][k][t];
+                }
                 keep[c] = v;
+                zkeep[c] = z;
             }
         }
     }
+}
+
+// The stand-alone D_W: x = own - kappa acc in units of 2^ex, three bits finer than
+// the solver's (bf_dw) because x goes out as doubles and needs no spare ones;
+// |x| < 2^63.  kappa >= BF_KAPPA_MIN, so that kappa acc has the larger unit.
+//   The error of x, about 0.3 units of 2^(ex + 3), belongs to the largest component
+// of the star; FP64 arithmetic has one of about 0.4 * 2^-53 of the terms that make
+// up a component.  Those are at least |own| + kappa sum |hop terms| (size): where
+// that is below 2^52 units for a component, the result is true and the site is
+// done in FP64.  Links that mix colours hardly ever leave such a component (2 in
+// 10^5 sites of Gaussian vectors at kappa 0.21, 5 in 10^4 at the worst kappa).  At
+// the line the errors are equal (root mean square 0.39 of 2^-53 of the terms in
+// both, unit links and components of different size), above it block fixed point
+// has the smaller one.
+constexpr double BF_KAPPA_MIN = 0.0625;
+constexpr int BF_FINE = 3;
+template <int N>
+__device__ __forceinline__ bool bf_dw_fine(const bfc own[N], int eown, const bfc acc[N], const unsigned size[N],
+                                           int eref, const BfScal &k, bfc x[N], int &ex) {
+    ex = eref + 4 + k.e + 64 - BF_FINE;
+    const int n = ex - eown; // >= 0
+    bool small = false;
+    auto part = [&](long long o, long long a, unsigned z) { // z: the size in the upper half
+        int h, l;
+        bf_split(a, h, l);
+        const long long mid = madw(h, k.l, madw(l, k.h, BF_HALF >> BF_FINE));
+        o = bf_shr(o, n);
+        const int oh = (int)(o >> 32);
+        small |= (unsigned)(oh ^ (oh >> 31)) + (__umulhi(z, (unsigned)k.h) << BF_FINE) < 1u << (52 + BF_FINE - 32);
+        return o - ((madw(h, k.h, 0) << BF_FINE) + (mid >> (32 - BF_FINE)));
+    };
+#pragma unroll
+    for (int c = 0; c < N; ++c)
+        x[c] = {part(own[c].x, acc[c].x, size[c] << 16), part(own[c].y, acc[c].y, size[c] & 0xffff0000u)};
+    return small;
 }
 // x = own - kappa acc in units of 2^eu, eu at least `least` (>= eown + 2, the
 // exponent of the block own); |x| < 2^60
@@ -437,11 +545,12 @@ __device__ __forceinline__ void bf_dw(const bfc own[N], int eown, const bfc acc[
     if (eref >= BF_BAD / 2) eu = BF_BAD;
 }
 
-// sites times columns up to which a stand-alone D_W is split over four threads
-// each (one vector of 4^4: 48 against 58 us; 98 304 on 12 vectors of 8^3x16: 110
-// against 97 us, there the SMs are full.  A solve's launches gained nothing: D_ov
-// on 3 vectors of 8^3x16 13.6 against 13.2 ms)
-constexpr size_t BF_SPLIT_MAX = 40000;
+// Sites times columns up to which a stand-alone D_W is split over four threads
+// each: 10 us against 20 for 256 (one vector of 4^4), 16.4 against 20.6 for 16 384,
+// 24.8 against 24.5 for 24 576, 26.7 against 22.8 for 32 768 (there the SMs are
+// full).  A solve's launches gained nothing from it: D_ov on 3 vectors of 8^3x16
+// 13.6 against 13.2 ms.
+constexpr size_t BF_SPLIT_MAX = 24000;
 // thread -> (site, column) of the block-fixed-point kernels: blocks of about a
 // hundred threads, so that small lattices reach every SM (24 576 sites and
 // columns are 384 blocks); 128 registers a thread

@@ -256,14 +256,14 @@ __global__ void __launch_bounds__(128) abi_to_bf_kernel(const double2 *__restric
     double2 d[12];
     bfc b[12];
     int x;
-    bool wide;
 #pragma unroll
     for (int c = 0; c < 12; ++c) d[c] = in[base + (size_t)c * B];
-    bf_from_double(d, b, x, wide);
+    const int span = bf_from_double(d, b, x);
 #pragma unroll
     for (int c = 0; c < 12; ++c) v[base + (size_t)c * B] = b[c];
-    // not finite, or components more than 2^40 apart: the sites that read it are done in FP64
-    e[i] = wide ? BF_BAD : x;
+    // not finite, or components 2^24 and more apart (3 in 10^6 sites of Gaussian
+    // vectors): the sites that read it are done in FP64 without a try
+    e[i] = bf_tag(span >= 24 ? BF_BAD : x, span >= 12);
 }
 
 // D_W at one site and column in FP64 (what block fixed point does not hold)
@@ -283,61 +283,166 @@ static __device__ __noinline__ void dw_site_fp64(const Geom &g, const double2 *_
     }
 }
 
-// one thread per site and column; bound by the integer pipe
+// x times 1, i, -1, -i for r = 0..3
+static __device__ __forceinline__ double2 turned(double2 x, int r) {
+    const double2 y = r & 1 ? make_double2(-x.y, x.x) : x;
+    return r & 2 ? make_double2(-y.x, -y.y) : y;
+}
+// The same by a whole warp: lane 3 k + a does colour row a of hop k, then the hops
+// are added in their order (the bits of dw_site_fp64).  An FP64 instruction takes a
+// warp as long for one lane as for 32: 110 of them instead of 960, 4 us instead of
+// 30, which every launch with one such site waited for.
+static __device__ __noinline__ void dw_site_fp64_warp(const Geom &g, const double2 *__restrict__ U,
+                                                      const double2 *__restrict__ in, double2 *__restrict__ out, int s,
+                                                      int B, int dagger, double kappa) {
+    const int lane = threadIdx.x & 31, k = min(lane / 3, 7), a = lane % 3, mu = k >> 1;
+    const bool back = k & 1;
+    const SiteCoords xc(g, s);
+    int n = g.n[0], st = g.stride[0], c = xc.x[0];
+    float bc = g.bcf[0];
+#pragma unroll
+    for (int m = 1; m < 4; ++m)
+        if (mu == m) {
+            n = g.n[m];
+            st = g.stride[m];
+            c = xc.x[m];
+            bc = g.bcf[m];
+        }
+    const bool edge = c == (back ? 0 : n - 1);
+    const int nb = back ? (edge ? s + (n - 1) * st : s - st) : (edge ? s - (n - 1) * st : s + st);
+    const int sg = (dagger != 0) != back ? 0 : 2; // the sign of gamma, as turns
+    // S_mu on the lower pair: (-i p3, -i p2), (-p3, p2), (-i p2, i p3), (p2, p3)
+    const int r0 = mu == 0 || mu == 2 ? 3 : mu == 1 ? 2 : 0, r1 = mu == 0 ? 3 : mu == 2 ? 1 : 0;
+    double2 w0 = make_double2(0, 0), w1 = w0;
+    const double2 *q = in + (size_t)nb * 12 * B, *ul = U + ((size_t)mu * g.V + (back ? nb : s)) * 9;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const double2 p2 = q[(size_t)(6 + b) * B], p3 = q[(size_t)(9 + b) * B];
+        const double2 h0 = cadd(q[(size_t)b * B], turned(mu < 2 ? p3 : p2, (r0 + sg) & 3));
+        const double2 h1 = cadd(q[(size_t)(3 + b) * B], turned(mu < 2 ? p2 : p3, (r1 + sg) & 3));
+        double2 u = ul[back ? b * 3 + a : a * 3 + b];
+        if (back) u.y = -u.y;
+        w0 = cfma(u, h0, w0);
+        w1 = cfma(u, h1, w1);
+    }
+    if (edge && bc < 0) {
+        w0 = cneg(w0);
+        w1 = cneg(w1);
+    }
+    // S_mu^dag: (i w1, i w0), (w1, -w0), (i w0, -i w1), (w0, w1)
+    const double2 t[4] = {w0, w1, turned(mu < 2 ? w1 : w0, ((mu == 0 || mu == 2 ? 1 : 0) + sg) & 3),
+                          turned(mu < 2 ? w0 : w1, ((mu == 0 ? 1 : mu == 1 ? 2 : mu == 2 ? 3 : 0) + sg) & 3)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        double2 acc = make_double2(0, 0);
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+            acc.x += __shfl_sync(0xffffffffu, t[i].x, 3 * h + a);
+            acc.y += __shfl_sync(0xffffffffu, t[i].y, 3 * h + a);
+        }
+        if (lane < 3) {
+            const size_t o = ((size_t)s * 12 + 3 * i + a) * B;
+            double2 v = in[o];
+            v.x -= kappa * acc.x;
+            v.y -= kappa * acc.y;
+            out[o] = v;
+        }
+    }
+}
+// most sites of a warp that it does one after the other (eight take as long as 32 threads side by side)
+constexpr int FP64_WARP_MAX = 8;
+
+// One thread per site and column; bound by the integer pipe (8^3x16: 51 us for 12
+// columns, 3.94 ms for 1000; with 128 registers and four blocks an SM 57 us and
+// 4.02 ms, the sizes of the terms spill).  Sites whose star
+// holds a bad block, and those where bf_dw_fine finds a component too small for
+// the common unit, are done in FP64 (`in` is read there: it may not overlap out).
+// A warp whose sites look uneven for the most part does not try (fields of sites or
+// components of very different size: 243 to 250 us a call on 12 columns of 8^3x16
+// with links that do not mix them, 265 to 271 with both).
 template <bool DAG>
-__global__ void __launch_bounds__(128, 4)
+__global__ void __launch_bounds__(128, 3)
     dslash_bf_kernel(Geom g, const int4 *__restrict__ Ubf, const double2 *__restrict__ U64, const bfc *__restrict__ v,
                      const int *__restrict__ e, const double2 *__restrict__ in, double2 *__restrict__ out, int B,
                      BfScal ks, double kappa) {
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (i >= (long)g.V * B) return;
-    const int s = (int)(i / B), j = (int)(i % B);
+    const bool on = i < (long)g.V * B;
+    const int s = on ? (int)(i / B) : 0, j = on ? (int)(i % B) : 0;
     const BfOff<0> off{g.V, B};
     const int one = opaque_one();
-    bfc acc[12], own[12];
-    int eown, eref, eu;
-    bf_wilson<DAG>(g, Ubf, v + j, e + j, off, s, one, acc, eown, eref);
-    if (eref >= BF_BAD / 2) {
-        dw_site_fp64(g, U64, in + j, out + j, s, B, DAG, kappa);
+    const BfStar x(g, e + j, off, s);
+    const bool most = __popc(__ballot_sync(0xffffffffu, on && x.uneven)) >= 16;
+    bool fp64 = on && !x.alone && (most || x.bad());
+    if (on && !fp64) {
+        if (x.alone) {
+#pragma unroll
+            for (int c = 0; c < 12; ++c) out[j + off(s, c)] = in[j + off(s, c)];
+        } else {
+            bfc acc[12], own[12];
+            unsigned size[12];
+            int ex;
+            bf_hops<DAG>(x, g, Ubf, v + j, e + j, off, s, one, acc, size);
+#pragma unroll
+            for (int c = 0; c < 12; ++c) own[c] = v[j + off(s, c)];
+            fp64 = bf_dw_fine<12>(own, x.eown, acc, size, x.eref, ks, acc, ex);
+            if (!fp64)
+#pragma unroll
+                for (int c = 0; c < 12; ++c)
+                    out[j + off(s, c)] = make_double2(bf_double(acc[c].x, ex), bf_double(acc[c].y, ex));
+        }
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, fp64);
+    if (__popc(todo) > FP64_WARP_MAX) {
+        if (fp64) dw_site_fp64(g, U64, in + j, out + j, s, B, DAG, kappa);
         return;
     }
-#pragma unroll
-    for (int c = 0; c < 12; ++c) own[c] = v[j + off(s, c)];
-    bf_dw<12>(own, eown, acc, eref, ks, eown + 2, one, acc, eu);
-#pragma unroll
-    for (int c = 0; c < 12; ++c)
-        out[j + off(s, c)] = make_double2(bf_double(acc[c].x, eu), bf_double(acc[c].y, eu));
+    for (; todo; todo &= todo - 1) {
+        const int from = __ffs(todo) - 1, sf = __shfl_sync(0xffffffffu, s, from), jf = __shfl_sync(0xffffffffu, j, from);
+        dw_site_fp64_warp(g, U64, in + jf, out + jf, sf, B, DAG, kappa);
+    }
 }
-// four threads per site and column (bf_wilson_split), 32 of those per block: up to
+// four threads per site and column (bf_hops_split), 32 of those per block: up to
 // BF_SPLIT_MAX of them, where one thread's eight hops in a row set the time
 template <bool DAG>
 __global__ void __launch_bounds__(128, 4)
     dslash_bf_split_kernel(Geom g, const int4 *__restrict__ Ubf, const double2 *__restrict__ U64,
                            const bfc *__restrict__ v, const int *__restrict__ e, const double2 *__restrict__ in,
                            double2 *__restrict__ out, int B, BfScal ks, double kappa) {
-    __shared__ bfc sm[4][6][32];
-    const int q = threadIdx.x / 32;
-    const long i = blockIdx.x * 32l + threadIdx.x % 32;
+    __shared__ BfSplit<32> sm;
+    __shared__ int fp64[32];
+    const int q = threadIdx.x / 32, t = threadIdx.x % 32;
+    const long i = blockIdx.x * 32l + t;
     const bool on = i < (long)g.V * B;
     const int s = on ? (int)(i / B) : 0, j = on ? (int)(i % B) : 0;
     const BfOff<0> off{g.V, B};
     const int one = opaque_one();
+    const BfStar x(g, e + j, off, s);
+    const bool todo64 = on && !x.alone && x.bad(), hop = on && !x.alone && !todo64;
+    if (q == 0) fp64[t] = todo64;
     bfc acc[3], own[3];
-    int eown, eref, eu;
-    bf_wilson_split<DAG, 32>(g, Ubf, v + j, e + j, off, s, on, one, sm, acc, eown, eref);
-    if (!on) return;
-    if (eref >= BF_BAD / 2) {
-        if (q == 0) dw_site_fp64(g, U64, in + j, out + j, s, B, DAG, kappa);
-        return;
+    unsigned size[3];
+    int ex;
+    bf_hops_split<DAG, 32>(x, g, Ubf, v + j, e + j, off, s, hop, one, sm, acc, size);
+    if (hop) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) own[c] = v[j + off(s, 3 * q + c)];
+        if (bf_dw_fine<3>(own, x.eown, acc, size, x.eref, ks, acc, ex)) fp64[t] = 1;
     }
+    __syncthreads();
+    if (on && !fp64[t])
 #pragma unroll
-    for (int c = 0; c < 3; ++c) own[c] = v[j + off(s, 3 * q + c)];
-    bf_dw<3>(own, eown, acc, eref, ks, eown + 2, one, acc, eu);
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-        out[j + off(s, 3 * q + c)] = make_double2(bf_double(acc[c].x, eu), bf_double(acc[c].y, eu));
+        for (int c = 0; c < 3; ++c) {
+            const size_t o = j + off(s, 3 * q + c);
+            out[o] = x.alone ? in[o] : make_double2(bf_double(acc[c].x, ex), bf_double(acc[c].y, ex));
+        }
+    unsigned todo = __ballot_sync(0xffffffffu, fp64[t] != 0); // the same in every warp
+    for (int k = 0; todo; todo &= todo - 1, ++k) { // the warps take turns
+        const int from = __ffs(todo) - 1, sf = __shfl_sync(0xffffffffu, s, from), jf = __shfl_sync(0xffffffffu, j, from);
+        if ((k & 3) == q) dw_site_fp64_warp(g, U64, in + jf, out + jf, sf, B, DAG, kappa);
+    }
 }
 
+bool bf_dslash(double kappa) { return kappa >= BF_KAPPA_MIN; }
 size_t bf_field_bytes(int V, int B) { return (size_t)V * B * (12 * sizeof(bfc) + sizeof(int)); }
 
 void launch_abi_to_bf(const double *in, void *field, int V, int B, cudaStream_t st) {
@@ -468,7 +573,7 @@ extern "C" int smpq_dslash_noalloc(smpq_ctx *ctx, const double *in, double *out,
         const int BC = 1;
         const bool apart = in + 2 * n <= out || out + 2 * n <= in;
         // (a block-fixed-point field is a 48th larger than the FP64 one: it fits where two of those do)
-        if (precision == SMPQ_FP64 && apart) {
+        if (precision == SMPQ_FP64 && apart && bf_dslash(ctx->opt.kappa)) {
             launch_abi_to_bf(in, scratch, ctx->V, B, st);
             launch_dslash_bf(ctx->geom, ctx->Ubf.p, ctx->U64.p, scratch, in, out, B, dagger, ctx->opt.kappa, st);
         } else if (precision == SMPQ_FP32) { // (the input is copied before anything is written)

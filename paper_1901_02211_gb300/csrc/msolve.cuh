@@ -886,13 +886,12 @@ __global__ void __launch_bounds__(BfMap<BC>::THREADS)
         double2 b[12];
         bfc v[12];
         int e;
-        bool wide;
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
             b[c] = source_at<BC>(src, g.V, s, c, j, base + ((size_t)s * 12 + c) * BC);
             acc += b[c].x * b[c].x + b[c].y * b[c].y;
         }
-        bf_from_double(b, v, e, wide);
+        bf_from_double(b, v, e);
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
             r.v[base + off(s, c)] = v[c];

@@ -122,7 +122,9 @@ template <typename T> void launch_dslash(const Geom &g, const void *U, const voi
 
 // D_W on the caller's layout [V][12][B]: in converted to a block-fixed-point
 // field (bf_field_bytes) and then out (not overlapping in) = D_W in; the FP32 one
-// takes a field of 12 V B float2 (out may be in)
+// takes a field of 12 V B float2 (out may be in).  For kappa below
+// BF_KAPPA_MIN (bf_dslash false) D_W is done in FP64 arithmetic.
+bool bf_dslash(double kappa);
 size_t bf_field_bytes(int V, int B);
 void launch_abi_to_bf(const double *in, void *field, int V, int B, cudaStream_t st);
 void launch_dslash_bf(const Geom &g, const void *Ubf, const void *U64, const void *field, const double *in,
