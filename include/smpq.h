@@ -271,9 +271,9 @@ int smpq_time_dslash(smpq_ctx *ctx, int B, int dagger, int precision, int reps, 
  * see every allocation (a framework's caching allocator), or latency-critical
  * loops where cudaMalloc/cudaFree would synchronise the device.  This call
  * allocates nothing: in and out are caller-owned DEVICE buffers in the layout
- * of smpq_dslash, and the kernel's scratch (tiled copies of in and out) lives
- * in a file-scope device array of 32 MiB that every GPU which loads the
- * library holds until the process exits.
+ * of smpq_dslash (they may overlap), and the kernel's scratch (copies of in and
+ * out) lives in a file-scope device array of 32.4 MiB that every GPU which loads
+ * the library holds until the process exits.
  *   - Limit: 2 * V * 12 * B * e bytes <= 32 MiB, e = 16 (FP64) or 8 (FP32);
  *     larger requests return SMPQ_EINVAL with the sizes in smpq_last_error.
  *   - The first call on a device looks up the device address of the scratch

@@ -1091,25 +1091,23 @@ int smpq_dslash(smpq_ctx *ctx, const double *in, double *out, int B, int dagger,
     cudaStream_t st = ctx->stream;
     const size_t n = (size_t)ctx->V * 12 * B;
     const size_t fb = dslash_field_bytes(ctx, precision, B);
-    // host buffers: staged copies of in and out; device: the caller's
+    // scratch: a copy of in (host buffers, and where block fixed point would write
+    // over the in that its FP64 sites read), of out (host buffers), the fields
     const bool bf = precision == SMPQ_FP64 && bf_dslash(ctx->opt.kappa);
-    const size_t bfb = bf ? bf_field_bytes(ctx->V, B) : 0;
-    const bool apart = !on_device || in + 2 * n <= out || out + 2 * n <= in;
-    const size_t stage = on_device ? 0 : n * 16;
-    if ((rc = ensure(ctx, ctx->ws[W_SRC], 2 * stage + std::max(2 * fb, bfb)))) return rc;
-    double *abi = (double *)ctx->ws[W_SRC].p + stage / 8;
-    char *tin = (char *)ctx->ws[W_SRC].p + 2 * stage, *tout = tin + fb;
-    const double *din = in;
-    if (!on_device) {
-        cudaMemcpyAsync(ctx->ws[W_SRC].p, in, n * 16, cudaMemcpyHostToDevice, st);
-        din = (const double *)ctx->ws[W_SRC].p;
-    }
+    const bool apart = in + 2 * n <= out || out + 2 * n <= in;
+    const size_t copy = !on_device || (bf && !apart) ? n * 16 : 0, res = on_device ? 0 : n * 16;
+    const size_t fields = std::max(2 * fb, bf ? bf_field_bytes(ctx->V, B) : 0);
+    if ((rc = ensure(ctx, ctx->ws[W_SRC], copy + res + fields))) return rc;
+    double *abi = (double *)ctx->ws[W_SRC].p;
+    char *tin = (char *)abi + copy + res, *tout = tin + fb;
+    if (copy) cudaMemcpyAsync(abi, in, n * 16, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
+    const double *din = copy ? abi : in;
+    double *dout = on_device ? out : abi + res / 8;
     const void *U = dslash_links(ctx, precision);
-    double *dout = on_device ? out : abi;
-    if (bf && apart) {
+    if (bf) {
         launch_abi_to_bf(din, tin, ctx->V, B, st);
         launch_dslash_bf(ctx->geom, ctx->Ubf.p, U, tin, din, dout, B, dagger, ctx->opt.kappa, st);
-    } else if (precision == SMPQ_FP64) { // small kappa or overlapping fields: through copies of both
+    } else if (precision == SMPQ_FP64) { // small kappa: through copies of both
         launch_to_tiled<double>(din, tin, ctx->V, B, 1, st);
         launch_dslash<double>(ctx->geom, U, tin, tout, B, 1, dagger, ctx->opt.kappa, st);
         launch_from_tiled<double>(tout, dout, ctx->V, B, 1, st);
@@ -1120,7 +1118,7 @@ int smpq_dslash(smpq_ctx *ctx, const double *in, double *out, int B, int dagger,
         launch_dslash_half(precision, ctx->geom, U, tin, tout, B, dagger, ctx->opt.kappa, st);
         launch_from_half(precision, tout, dout, ctx->V, B, st);
     }
-    if (!on_device) cudaMemcpyAsync(out, abi, n * 16, cudaMemcpyDeviceToHost, st);
+    if (!on_device) cudaMemcpyAsync(out, dout, n * 16, cudaMemcpyDeviceToHost, st);
     cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_check(ctx, e, "dslash");
     return cuda_check(ctx, cudaGetLastError(), "dslash launch");

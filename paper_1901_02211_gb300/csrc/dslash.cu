@@ -514,7 +514,10 @@ void launch_dslash_fp32_abi(const Geom &g, const void *U, const double *in, void
 // library's device code is loaded on a GPU and stays reserved on every GPU that
 // loads the library until the process exits.
 #define SMPQ_NOALLOC_SCRATCH_BYTES (32u << 20)
-static __device__ __align__(256) unsigned char g_noalloc_scratch[SMPQ_NOALLOC_SCRATCH_BYTES];
+// (the limit counts two fields; a block-fixed-point field is a 48th larger than an
+// FP64 one)
+static __device__ __align__(256) unsigned char
+    g_noalloc_scratch[SMPQ_NOALLOC_SCRATCH_BYTES + SMPQ_NOALLOC_SCRATCH_BYTES / 96 + 256];
 
 #include <mutex>
 
@@ -572,10 +575,14 @@ extern "C" int smpq_dslash_noalloc(smpq_ctx *ctx, const double *in, double *out,
         char *tin = (char *)scratch, *tout = (char *)scratch + half;
         const int BC = 1;
         const bool apart = in + 2 * n <= out || out + 2 * n <= in;
-        // (a block-fixed-point field is a 48th larger than the FP64 one: it fits where two of those do)
-        if (precision == SMPQ_FP64 && apart && bf_dslash(ctx->opt.kappa)) {
-            launch_abi_to_bf(in, scratch, ctx->V, B, st);
-            launch_dslash_bf(ctx->geom, ctx->Ubf.p, ctx->U64.p, scratch, in, out, B, dagger, ctx->opt.kappa, st);
+        if (precision == SMPQ_FP64 && bf_dslash(ctx->opt.kappa)) {
+            const double *din = in;
+            if (!apart) { // a copy of what the sites done in FP64 read
+                cudaMemcpyAsync(tin, in, n * sizeof(double2), cudaMemcpyDeviceToDevice, st);
+                din = (const double *)tin;
+            }
+            launch_abi_to_bf(din, tout, ctx->V, B, st);
+            launch_dslash_bf(ctx->geom, ctx->Ubf.p, ctx->U64.p, tout, din, out, B, dagger, ctx->opt.kappa, st);
         } else if (precision == SMPQ_FP32) { // (the input is copied before anything is written)
             launch_dslash_fp32_abi(ctx->geom, ctx->U32.p, in, scratch, out, B, dagger, ctx->opt.kappa, st);
         } else {

@@ -105,3 +105,47 @@ def test_dslash_components(S, links, dims, B, kappa):
             terms = _terms(U, x, dims, kappa)
             for dag in (False, True):
                 _check(s.dslash(x, dagger=dag), _ref(U, x, dims, kappa, bc, dag), terms)
+
+
+@pytest.mark.parametrize("B", [1, 3, 6])
+@pytest.mark.parametrize("shift", [0, 1, 1000])
+def test_dslash_overlapping_buffers(S, shift, B):
+    """out over in, or part of it: the bits of the call on two buffers, also where
+    sites are done in FP64 from in."""
+    import torch
+    from paper_1901_02211_gb300 import Session
+    rng = np.random.default_rng(19)
+    dims, V = (4, 6, 4, 8), 768
+    n = V * 12 * B
+    psi = random_spinor(rng, V, B)
+    psi[:40] *= np.array([1, 1e-7, 1])[None, None, :, None]
+    psi[300, 0, 0, 0] = np.nan
+    with Session() as s:
+        s.load_gauge(dims, _links("diagonal", rng, V))
+        for prec in (S.SMPQ_FP64, S.SMPQ_FP32):
+            for call in (S.smpq_dslash, S.smpq_dslash_noalloc):
+                d = torch.from_numpy(psi).cuda()
+                want = torch.empty_like(d)
+                call(s.ctx, d, want, B, False, prec)
+                room = torch.zeros(n + shift, dtype=torch.complex128, device="cuda")
+                for i, o in ((room[:n], room[shift:]), (room[shift:], room[:n])):
+                    i, o = i.view(V, 4, 3, B), o.view(V, 4, 3, B)
+                    i.copy_(d)
+                    call(s.ctx, i, o, B, False, prec)
+                    assert torch.equal(torch.view_as_real(o).view(torch.int64), torch.view_as_real(want).view(torch.int64))
+
+
+def test_noalloc_in_place_at_its_limit(S):
+    """The largest field that fits the scratch, in place (copy and blocks side by side)."""
+    import torch
+    from paper_1901_02211_gb300 import Session
+    rng = np.random.default_rng(23)
+    dims, V, B = (4, 4, 4, 4), 256, (32 << 20) // (2 * 256 * 12 * 16)
+    psi = random_spinor(rng, V, B)
+    with Session() as s:
+        s.load_gauge(dims, _links("haar", rng, V))
+        d = torch.from_numpy(psi).cuda()
+        want = torch.empty_like(d)
+        S.smpq_dslash(s.ctx, d, want, B)
+        S.smpq_dslash_noalloc(s.ctx, d, d, B)
+        assert torch.equal(torch.view_as_real(d), torch.view_as_real(want))
