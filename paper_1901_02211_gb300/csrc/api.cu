@@ -1092,11 +1092,12 @@ int smpq_dslash(smpq_ctx *ctx, const double *in, double *out, int B, int dagger,
     const size_t n = (size_t)ctx->V * 12 * B;
     const size_t fb = dslash_field_bytes(ctx, precision, B);
     // scratch: a copy of in (host buffers, and where block fixed point would write
-    // over the in that its FP64 sites read), of out (host buffers), the fields
+    // over the in that its FP64 sites read), of out (the same, host buffers; the
+    // other formats read in no more when they write it), the fields
     const bool bf = precision == SMPQ_FP64 && bf_dslash(ctx->opt.kappa);
     const bool apart = in + 2 * n <= out || out + 2 * n <= in;
-    const size_t copy = !on_device || (bf && !apart) ? n * 16 : 0, res = on_device ? 0 : n * 16;
-    const size_t fields = std::max(2 * fb, bf ? bf_field_bytes(ctx->V, B) : 0);
+    const size_t copy = !on_device || (bf && !apart) ? n * 16 : 0, res = !on_device && bf ? n * 16 : 0;
+    const size_t fields = bf ? bf_field_bytes(ctx->V, B) : precision == SMPQ_FP32 ? fb : 2 * fb;
     if ((rc = ensure(ctx, ctx->ws[W_SRC], copy + res + fields))) return rc;
     double *abi = (double *)ctx->ws[W_SRC].p;
     char *tin = (char *)abi + copy + res, *tout = tin + fb;

@@ -149,3 +149,21 @@ def test_noalloc_in_place_at_its_limit(S):
         S.smpq_dslash(s.ctx, d, want, B)
         S.smpq_dslash_noalloc(s.ctx, d, d, B)
         assert torch.equal(torch.view_as_real(d), torch.view_as_real(want))
+
+
+@pytest.mark.parametrize("prec,copies", [("FP64", 3.1), ("FP32", 2.0), ("FP16N", 1.6), ("BF16N", 1.6)])
+def test_dslash_host_buffers_scratch(S, prec, copies):
+    """Device memory that a call on host buffers takes: a copy of the vectors and the
+    fields in the format's size (FP64: input, blocks and output), in copies of the
+    vectors; 4 MiB for the allocator's rounding."""
+    import torch
+    from paper_1901_02211_gb300 import Session
+    rng = np.random.default_rng(29)
+    dims, V, B = (8, 8, 8, 16), 8192, 16
+    psi = random_spinor(rng, V, B)
+    with Session() as s:
+        s.load_gauge(dims, _links("unit", rng, V))
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        s.dslash(psi, precision=getattr(S, "SMPQ_" + prec))
+        assert free - torch.cuda.mem_get_info()[0] <= copies * psi.nbytes + (4 << 20)
