@@ -1435,9 +1435,10 @@ __device__ __forceinline__ void shift_scalars(const Scal &sc, int k, int i, int 
 }
 // The weights of a chunk of n iterations, one thread per shift and column of a
 // lattice (columns j0 <= j < j0 + Bl): hz <- c_i zeta_k S_{k+1}, ho <- zeta_k
-// P_{k+1} (as two FP32 values); v0 <- c_i S_0, d0 <- P_0.
+// P_{k+1} (packed: as two FP32 values, for k_hist_p<.., true>); v0 <- c_i S_0,
+// d0 <- P_0.
 __global__ void k_hist_w(int n, int nshift, int B, int j0, int Bl, const ShiftParams *__restrict__ sp, Scal sc,
-                         double *__restrict__ v0, double *__restrict__ d0) {
+                         double *__restrict__ v0, double *__restrict__ d0, bool packed) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nshift * Bl) return;
     const int i = t / Bl, j = j0 + t % Bl;
@@ -1450,7 +1451,7 @@ __global__ void k_hist_w(int n, int nshift, int B, int j0, int Bl, const ShiftPa
         double a, b, z;
         shift_scalars(sc, k, i, j, nshift, B, a, b, z);
         sc.hz[o] = c * (z * S);
-        sc.ho[o] = hi_lo(z * P);
+        sc.ho[o] = packed ? hi_lo(z * P) : z * P;
         S = fma(b, S, a);
         P *= b;
     }
@@ -1571,9 +1572,11 @@ template <int BC> static dim3 hist_grid(const HistLat &L) {
 
 // p_i = P_0 p_i + sum_k zeta_k P_{k+1} r_k for every shift after a chunk of
 // FP64-accurate iterations.  Into ps (FP64; more such iterations follow): FP64
-// sums.  Into ps32 (the mixed solve's switch to FP32): float-float sums (48
-// bits, re and im packed: 12 FP32 instructions of 2 cycles for the two FP64
-// ones of 66), rounded to FP32 at the end.
+// weights and sums.  Into ps32 (the mixed solve's switch to FP32): float-float
+// ones (48 bits, re and im packed: 12 FP32 instructions of 2 cycles for the two
+// FP64 ones of 66), rounded to FP32 at the end.  The weights then fall like
+// (|r_n| / |r_k|)^2: one below the FP32 range belongs to a term that far below
+// the last ones.
 template <typename C, int BC, bool F32>
 __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_p(HistLat L, const double *__restrict__ hp,
                                                                  const double *__restrict__ d0,
@@ -1611,20 +1614,20 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_p(HistLat L, cons
 #pragma unroll
                 for (int k = 0; k < HK; ++k) {
                     // every shift's zeta is 0 where the column was idle, and only there is the slot unset
-                    if (__double2loint(sm[k][0][T.jj]) == 0) continue;
+                    const double w0 = sm[k][0][T.jj];
+                    if (F32 ? __double2loint(w0) == 0 : w0 == 0) continue;
                     const C v = ((const C *)L.h)[(k0 + k) * L.stride + T.e[q]];
 #pragma unroll
                     for (int g = 0; g < NG; ++g) {
                         const double w = sm[k][g][T.jj];
-                        const float wh = __int_as_float(__double2loint(w)), wl = __int_as_float(__double2hiint(w));
                         if constexpr (F32 && std::is_same<C, df64c>::value) {
+                            const float wh = __int_as_float(__double2loint(w)), wl = __int_as_float(__double2hiint(w));
                             ff_acc2(sh[g], sl[g], f2b(wh), f2b(wl), make_float2(v.x.hi, v.y.hi),
                                     make_float2(v.x.lo, v.y.lo));
                         } else if constexpr (!F32) {
                             const double2 d = hist_value(v);
-                            const double wd = exact_d(wh) + exact_d(wl);
-                            acc[g].x = fma(wd, d.x, acc[g].x);
-                            acc[g].y = fma(wd, d.y, acc[g].y);
+                            acc[g].x = fma(w, d.x, acc[g].x);
+                            acc[g].y = fma(w, d.y, acc[g].y);
                         }
                     }
                 }
@@ -2334,7 +2337,7 @@ template <int BC> struct Solve {
         if (next == 1 && (rc = hist_dirs(W_PS, sizeof(double2)))) return rc;
         if (next == 2 && (rc = hist_dirs(W_PS32, sizeof(float2)))) return rc;
         for (int l = 0; l < nl; ++l)
-            k_hist_w<<<(nshift * Bl[l] + 127) / 128, 128, 0, st>>>(n, nshift, B, j0[l], Bl[l], spd + l, sc, hv0, hd0);
+            k_hist_w<<<(nshift * Bl[l] + 127) / 128, 128, 0, st>>>(n, nshift, B, j0[l], Bl[l], spd + l, sc, hv0, hd0, next == 2);
         k_hist_sum<<<(unsigned)(((size_t)(n + 1) * B + 255) / 256), 256, 0, st>>>(n, nshift, B, sc.hz, hv0, hw);
         for (int l = 0; l < nl; ++l) {
             HistLat L = hist_lat(l);
