@@ -1663,11 +1663,16 @@ __global__ void k_hist_coef(int n, int nshift, int B, int j0, int Bl, const Shif
 
 // A chunk of FP32 iterations: y += c_i alpha_i p_i, p_i = zeta r + beta p_i for
 // every shift, in the order of the iterations, the directions in registers.
-// EXACT: y in FP64 all through (SMPQ_FP32 and the half storage, where y starts
-// here).  Else (the mixed solve, whose FP32 share of y is below the switch
-// residual) the chunk's share is summed in float-float, 48 bits of a thousandth,
-// and added to y in FP64: 10 packed FP32 instructions a value instead of FP64
-// ones of 66 cycles.  Bound by those.
+// EXACT: y in FP64 all through (hist_exact).  Else the chunk's share is summed in
+// float-float and added to y in FP64: 10 packed FP32 instructions a value instead
+// of FP64 ones of 66 cycles.  Bound by those.
+//   Float-float coefficients and sums round at about 2^-48 of the share, FP64 ones at
+// 2^-53 of y in every addition.  In the mixed solve the share is what is left of y
+// below the switch residual theta (times a factor of order 1): for theta up to 2^-8
+// (the default is 1e-3) its rounding is no larger than FP64's.  Above that, and where
+// y starts here (SMPQ_FP32 and the half storage), the sums are FP64.
+constexpr double HIST_FF_THETA = 1.0 / 256;
+inline bool hist_exact(int prec, double theta) { return prec != SMPQ_MIXED || theta > HIST_FF_THETA; }
 template <int BC, bool EXACT>
 __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_run(HistLat L, const double *__restrict__ ca,
                                                                    const float4 *__restrict__ ct,
@@ -2355,7 +2360,7 @@ template <int BC> struct Solve {
     // the end of a chunk of FP32 iterations
     int hist_flush32(bool last) {
         std::vector<Buf> &ws = ctx->ws;
-        const bool exact = in[0].spec->prec != SMPQ_MIXED;
+        const bool exact = hist_exact(in[0].spec->prec, ctx->opt.switch_residual);
         int rc;
         if (!last && (rc = hist_dirs(W_PS32, sizeof(float2)))) return rc;
         for (int l = 0; l < nl; ++l) {

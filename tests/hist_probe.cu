@@ -18,8 +18,9 @@ template <typename T> struct Dev {
 
 // n iterations, nshift shifts; zn, zo [n][nshift][12], alpha, beta [n][12], c
 // [nshift]; r [n][ne], ps [nshift][ne], y [ne] with ne = 144 n_sup complex numbers.
-// A chunk of FP64 iterations: y and ps.
-extern "C" int hist_probe(int n, int nshift, int n_sup, const double *c, const double *zn,
+// fp32 = 0: a chunk of FP64 iterations (y and ps); 1: of FP32 ones, r and ps rounded
+// to FP32 first, y by the sums that a mixed solve with this switch residual takes.
+extern "C" int hist_probe(int fp32, double theta, int n, int nshift, int n_sup, const double *c, const double *zn,
                           const double *zo, const double *alpha, const double *beta, const double2 *r, double2 *ps,
                           double2 *y) {
     constexpr int B = 12;
@@ -30,8 +31,13 @@ extern "C" int hist_probe(int n, int nshift, int n_sup, const double *c, const d
     Dev<ShiftParams> dsp(&sp, 1);
     Dev<double> hz(zn, rows), ho(zo, rows), hal(alpha, (size_t)n * B), hbe(beta, (size_t)n * B);
     Dev<double> hw(nullptr, (size_t)(n + 1) * B), v0(nullptr, nshift * B), d0(nullptr, nshift * B);
+    Dev<float4> ct(nullptr, rows);
     Dev<int> cls(nullptr, B);
     Dev<double2> dy(y, ne), dps(ps, nshift * ne), dr(r, n * ne);
+    std::vector<float2> r32(n * ne), p32(nshift * ne);
+    for (size_t i = 0; i < n * ne; ++i) r32[i] = make_float2((float)r[i].x, (float)r[i].y);
+    for (size_t i = 0; i < nshift * ne; ++i) p32[i] = make_float2((float)ps[i].x, (float)ps[i].y);
+    Dev<float2> dr32(r32.data(), n * ne), dp32(p32.data(), nshift * ne);
     Scal sc{};
     sc.hz = hz.p;
     sc.ho = ho.p;
@@ -48,12 +54,19 @@ extern "C" int hist_probe(int n, int nshift, int n_sup, const double *c, const d
     L.n = n;
     const dim3 grid = hist_grid<B>(L);
     const int TH = TileMap<B>::THREADS;
-    L.h = dr.p;
-    k_hist_w<<<(nshift * B + 127) / 128, 128>>>(n, nshift, B, 0, B, dsp.p, sc, v0.p, d0.p, false);
-    k_hist_sum<<<(unsigned)(((size_t)(n + 1) * B + 255) / 256), 256>>>(n, nshift, B, hz.p, v0.p, hw.p);
-    k_hist_y<double2, B><<<(unsigned)((ne + 255) / 256), 256>>>(L, hw.p, v0.p, dps.p, dy.p);
-    k_hist_p<double2, B, false><<<grid, TH>>>(L, ho.p, d0.p, dps.p, nullptr);
-    dps.get(ps);
+    if (fp32) {
+        L.h = dr32.p;
+        k_hist_coef<<<(unsigned)((rows + 255) / 256), 256>>>(n, nshift, B, 0, B, dsp.p, sc, ct.p);
+        if (hist_exact(SMPQ_MIXED, theta)) k_hist_run<B, true><<<grid, TH>>>(L, ho.p, ct.p, dp32.p, dy.p, true);
+        else k_hist_run<B, false><<<grid, TH>>>(L, ho.p, ct.p, dp32.p, dy.p, true);
+    } else {
+        L.h = dr.p;
+        k_hist_w<<<(nshift * B + 127) / 128, 128>>>(n, nshift, B, 0, B, dsp.p, sc, v0.p, d0.p, false);
+        k_hist_sum<<<(unsigned)(((size_t)(n + 1) * B + 255) / 256), 256>>>(n, nshift, B, hz.p, v0.p, hw.p);
+        k_hist_y<double2, B><<<(unsigned)((ne + 255) / 256), 256>>>(L, hw.p, v0.p, dps.p, dy.p);
+        k_hist_p<double2, B, false><<<grid, TH>>>(L, ho.p, d0.p, dps.p, dp32.p);
+        dps.get(ps);
+    }
     dy.get(y);
     return (int)cudaDeviceSynchronize();
 }

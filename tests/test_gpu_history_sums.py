@@ -27,11 +27,11 @@ def probe(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     f = ctypes.CDLL(lib).hist_probe
 
-    def call(c, zn, zo, alpha, beta, r, ps, y):
+    def call(fp32, theta, c, zn, zo, alpha, beta, r, ps, y):
         n, nshift = zn.shape[:2]
         ps, y = ps.copy(), y.copy()
         ptr = [np.ascontiguousarray(a).ctypes.data_as(ctypes.c_void_p) for a in (c, zn, zo, alpha, beta, r)]
-        rc = f(n, nshift, r.shape[1] // 144, *ptr,
+        rc = f(int(fp32), ctypes.c_double(theta), n, nshift, r.shape[1] // 144, *ptr,
                ps.ctypes.data_as(ctypes.c_void_p), y.ctypes.data_as(ctypes.c_void_p))
         assert rc == 0
         return y, ps
@@ -60,7 +60,7 @@ def test_directions_after_one_iteration(probe, nshift, scale):
     r, ps, y = _fields(rng, 1, nshift, ne)
     zeta = scale * rng.uniform(0.5, 1, (1, nshift, 12))
     alpha, beta = rng.uniform(0.5, 1, (1, 12)), rng.uniform(0.5, 1, (1, 12))
-    _, got = probe(np.ones(nshift), zeta, zeta, alpha, beta, r / scale, ps, y)
+    _, got = probe(False, 0, np.ones(nshift), zeta, zeta, alpha, beta, r / scale, ps, y)
     col = _columns(ne)
     b, z = beta[0, col].astype(np.longdouble), zeta[0][:, col].astype(np.longdouble)
     rl = (r / scale)[0]
@@ -82,7 +82,7 @@ def test_chunk_of_fp64_iterations(probe, n, nshift):
     alpha, beta = rng.uniform(0.5, 1, (2, n, 12))
     zn[n // 2:, nshift - 1] = 0  # the last shift has converged
     c = rng.uniform(0.1, 1, nshift)
-    gy, gp = probe(c, zn, zo, alpha, beta, r, ps, y)
+    gy, gp = probe(False, 0, c, zn, zo, alpha, beta, r, ps, y)
     col = _columns(ne)
     L = np.longdouble
     p, s = ps.astype(np.clongdouble), y.astype(np.clongdouble)
@@ -101,3 +101,54 @@ def test_chunk_of_fp64_iterations(probe, n, nshift):
     bar = (6 * n + nshift + 4) * U
     assert (np.abs(gy.real - s.real) <= bar * sa).all()
     assert (np.abs(gp.real - p.real) <= bar * pa).all()
+
+
+@pytest.mark.parametrize("theta", [0.9, 0.5, 2.0 ** -7])
+@pytest.mark.parametrize("nshift", [1, 15])
+def test_share_of_fp32_iterations(probe, theta, nshift):
+    """y after one FP32 iteration of a mixed solve with a large switch residual, where
+    that iteration's share c alpha p is most of y: each term's coefficient rounds once,
+    its product with the sum once."""
+    rng = np.random.default_rng(5)
+    ne = 144 * 5
+    r, ps, _ = _fields(rng, 1, nshift, ne)
+    ps = ps.astype(np.complex64).astype(complex)
+    zeta = rng.uniform(0.5, 1, (1, nshift, 12))
+    alpha, beta = rng.uniform(0.5, 1, (2, 1, 12))
+    c = rng.uniform(0.1, 1, nshift)
+    got, _ = probe(True, theta, c, zeta, zeta, alpha, beta, r, ps, np.zeros(ne, complex))
+    a = c[:, None].astype(np.longdouble) * alpha[0, _columns(ne)]
+    for part in ("real", "imag"):
+        terms = a * getattr(ps, part)
+        err = np.abs(getattr(got, part) - terms.sum(0))
+        # alpha z / z rounds twice, times c once
+        assert (err <= (3 + nshift) * U * np.abs(terms).sum(0)).all()
+
+
+@pytest.mark.parametrize("n", [1, 7, 30])
+def test_share_below_a_small_switch_residual(probe, n):
+    """At the largest switch residual with float-float sums, y of that many times the
+    share: within the FP64 sums' own bound (an addition per shift and iteration)."""
+    rng = np.random.default_rng(n)
+    ne, nshift = 144 * 3, 14
+    r, ps, _ = _fields(rng, n, nshift, ne)
+    r, ps = (x.astype(np.complex64).astype(complex) for x in (r, ps))
+    zeta = np.broadcast_to(rng.uniform(0.5, 1, (1, nshift, 12)), (n, nshift, 12)).copy()
+    alpha, beta = rng.uniform(0.5, 1, (2, n, 12)) / n
+    c = rng.uniform(0.1, 1, nshift)
+    y = 256 * (rng.choice([-1, 1], ne) + 1j * rng.choice([-1, 1], ne)) * rng.uniform(1, 2, ne)
+    got, _ = probe(True, 2.0 ** -8, c, zeta, zeta, alpha, beta, r, ps, y)
+    col = _columns(ne)
+    s = y.astype(np.clongdouble)
+    p = ps.astype(np.complex64)
+    share = np.zeros(ne)
+    for k in range(n):
+        a = c[:, None].astype(np.longdouble) * alpha[k, col]
+        s = s + (a * p).sum(0)
+        share += (np.abs(a) * np.abs(p.real)).sum(0).astype(float)
+        z32, b32 = zeta[k][:, col].astype(np.float32), beta[k, col].astype(np.float32)
+        # the FP32 recurrence: product, then one fused multiply-add
+        zr = z32 * r[k].astype(np.complex64).real, z32 * r[k].astype(np.complex64).imag
+        p = ((b32.astype(float) * p.real + zr[0]).astype(np.float32)
+             + 1j * (b32.astype(float) * p.imag + zr[1]).astype(np.float32)).astype(np.complex64)
+    assert (np.abs(got.real - s.real) <= (n * nshift + 1) * U * (np.abs(y.real) + share)).all()
