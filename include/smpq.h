@@ -34,6 +34,10 @@
  * buffers are used in stream order on the context's stream and the call
  * synchronises that stream before returning); the library never frees caller
  * memory and owns every device allocation it makes (released by smpq_destroy).
+ * Workspaces are kept from call to call; the largest, the residual history of a
+ * multi-shift solve, takes at most a twelfth of the GPU's memory (or what npoles
+ * vectors on the solve's support take, if that is more), and less where the free
+ * memory is short.
  * A context is not thread-safe; use one context per host thread.
  */
 #ifndef SMPQ_H

@@ -296,9 +296,11 @@ size_t bytes_per_rhs(const smpq_ctx *ctx, int prec, int n_sup, int npoles) {
     size_t full = (size_t)ctx->V * 12 * per;
     // support: y and the residual history, or as much of that as the fields
     // take (a shorter history needs the shifted directions beside it)
-    const size_t want = (size_t)n_sup * 12 * hist_bytes_wanted(prec, ctx->opt.max_iter);
-    const size_t dirs = (size_t)n_sup * 12 * npoles * 16;
-    return full + (size_t)n_sup * 12 * 16 + std::min(want, std::max(full, dirs) + dirs);
+    const size_t slots = hist_bytes_wanted(prec, ctx->opt.max_iter);
+    const size_t want = (size_t)n_sup * 12 * slots, dirs = (size_t)n_sup * 12 * npoles * 16;
+    // and, per slot, the scalars of every shift
+    const size_t scalars = slots / (prec == SMPQ_FP64 ? 16 : 8) * (npoles * 32 + 24);
+    return full + (size_t)n_sup * 12 * 16 + std::min(want, std::max(full, dirs) + dirs) + scalars;
 }
 
 // kind 0: q^SMP(x) of Eq. 16; kind 1: SMP estimate of diag D_W^{-1}
@@ -814,6 +816,8 @@ int smpq_create(smpq_ctx **out, int device, void *stream, const smpq_options *op
     if (e == cudaSuccess) e = cudaEventCreate(&ctx->ev2);
     if (e == cudaSuccess) e = cudaEventCreate(&ctx->evA);
     if (e == cudaSuccess) e = cudaEventCreate(&ctx->evB);
+    size_t freeb = 0;
+    if (e == cudaSuccess) e = cudaMemGetInfo(&freeb, &ctx->mem_total);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete ctx;

@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <initializer_list>
 
 #include "bfp.cuh"
 #include "half.cuh"
@@ -2258,50 +2259,85 @@ template <int BC> struct Solve {
         return HF<HT>{v, (float *)(v + nfield)};
     }
 
-    // Capacity of the history for this solve: W_HIST as it is if that is enough,
-    // else grown to hist_bytes_wanted per support element, or to what half of
-    // the free memory holds (the directions p_i, which a chunk's end needs, are
-    // then set aside first).
+    // Capacity of the history for this solve: hist_bytes_wanted per support element,
+    // at most a twelfth of the GPU's memory or what the directions p_i take (a
+    // chunk's end needs them, so that the solve can go on with less).  The solve's
+    // fields and the directions come first: where the rest of the free memory does not
+    // hold the history as well, the directions are set aside at once and it takes
+    // three quarters of what is left then.
     int plan_history() {
         std::vector<Buf> &ws = ctx->ws;
+        Buf &hist = ws[W_HIST];
         const int prec = in[0].spec->prec;
-        const size_t eb = prec == SMPQ_FP64 || prec == SMPQ_MIXED ? sizeof(double2) : sizeof(float2);
-        const size_t least = 2 * eb;
-        size_t want = hist_bytes_wanted(prec, ctx->opt.max_iter);
-        if (ws[W_HIST].bytes < want * nsupf) {
-            size_t freeb = 0, totb = 0;
-            cudaMemGetInfo(&freeb, &totb);
-            const size_t half = (freeb + ws[W_HIST].bytes) / 2;
-            int rc;
-            if (want * nsupf > half) {
-                if ((eb == sizeof(double2) && (rc = hist_dirs(W_PS, sizeof(double2)))) ||
-                    (prec != SMPQ_FP64 && (rc = hist_dirs(W_PS32, sizeof(float2)))))
-                    return rc;
+        const bool fp64 = prec == SMPQ_FP64, both = prec == SMPQ_MIXED;
+        const size_t eb = fp64 || both ? sizeof(double2) : sizeof(float2);
+        const size_t dirs = (size_t)nshift * ((fp64 || both ? sizeof(double2) : 0) + (fp64 ? 0 : sizeof(float2)));
+        const size_t most = std::max(dirs, ctx->mem_total / 12 / nsupf / eb * eb);
+        size_t want = std::min(hist_bytes_wanted(prec, ctx->opt.max_iter), most);
+        const size_t fields = missing_fields();
+        if (hist.bytes < want * nsupf || fields > 0) {
+            auto room = [&]() { // free for the history, less a little for buffers of a few bytes a source
+                size_t freeb = 0, totb = 0;
                 cudaMemGetInfo(&freeb, &totb);
-                // what the solve's fields and y will still take is left alone
-                const size_t fields = field_bytes(prec), room = freeb + ws[W_HIST].bytes;
-                const size_t give = room > fields ? (room - fields) / 2 : 0;
-                want = std::min(want, std::max(least, give / nsupf / eb * eb));
+                const size_t rows = want / (fp64 ? sizeof(double2) : sizeof(float2));
+                const size_t need = missing_fields() + missing_dirs() + rows * nshift * B * 32;
+                const size_t have = (freeb + hist.bytes) / 64 * 63;
+                return have > need ? have - need : 0;
+            };
+            int rc;
+            const size_t r = room();
+            if (hist.bytes > r) release(hist);
+            if (want * nsupf > r) {
+                if ((eb == sizeof(double2) && (rc = hist_dirs(W_PS, sizeof(double2)))) ||
+                    (!fp64 && (rc = hist_dirs(W_PS32, sizeof(float2)))))
+                    return rc;
+                want = std::min(want, std::max(eb, room() / 4 * 3 / nsupf / eb * eb));
             }
-            if (ws[W_HIST].bytes < want * nsupf && (rc = ensure(ctx, ws[W_HIST], want * nsupf))) return rc;
-        } else {
-            want = ws[W_HIST].bytes / nsupf / eb * eb;
+            if (hist.bytes < want * nsupf && (rc = ensure(ctx, hist, want * nsupf))) return rc;
         }
-        hcap = std::min(want, hist_bytes_wanted(prec, ctx->opt.max_iter));
-        hrows = (int)(hcap / (prec == SMPQ_FP64 ? sizeof(double2) : sizeof(float2)));
+        hcap = want;
+        hrows = (int)(hcap / (fp64 ? sizeof(double2) : sizeof(float2)));
         return SMPQ_OK;
     }
-    // bytes of the solve's whole-lattice fields and y that are not allocated yet
-    size_t field_bytes(int prec) const {
-        const size_t full = (prec == SMPQ_FP32                           ? 4 * 8 + 2 * 16
-                             : prec == SMPQ_FP16N || prec == SMPQ_BF16N ? 2 * 5 + 2 * 8 + 2 * 16
-                             : prec == SMPQ_MIXED                       ? 4 * 16 + 4 * 8
-                                                                        : 5 * 16) *
-                            nfield;
-        size_t held = 0;
-        for (int w : {W_P, W_T, W_R, W_XLO, W_XHI, W_T64}) held += ctx->ws[w].bytes;
-        const size_t yb = nsupf * sizeof(double2), yh = ctx->ws[W_Y].bytes;
-        return (full > held ? full - held : 0) + (yb > yh ? yb - yh : 0);
+    size_t missing(int w, size_t bytes) const {
+        const size_t held = ctx->ws[w].bytes;
+        return bytes > held ? bytes - held : 0;
+    }
+    // bytes of the solve's whole-lattice fields and y that are not allocated yet (run())
+    size_t missing_fields() const {
+        const size_t nf = nfield, d = nf * sizeof(double2), f = nf * sizeof(float2), hf = nf * 4 + nf / 12 * 4 + 256;
+        size_t m = missing(W_Y, nsupf * sizeof(double2));
+        if (in[0].spec->full_support) m += missing(W_OUT, d);
+        auto add = [&](size_t b, std::initializer_list<int> l) {
+            for (int w : l) m += missing(w, b);
+        };
+        switch (in[0].spec->prec) {
+        case SMPQ_FP64:
+            add(d + nf / 12 * sizeof(int), {W_P, W_T, W_R});
+            if (ctx->opt.true_residual) add(d, {W_XHI, W_T64});
+            break;
+        case SMPQ_MIXED:
+            add(d, {W_P, W_T, W_R});
+            if (ctx->opt.true_residual) add(d, {W_XHI});
+            add(4 * f, {W_XLO});
+            break;
+        case SMPQ_FP32:
+            add(f, {W_P, W_T, W_R, W_XLO});
+            add(d, {W_XHI, W_T64});
+            break;
+        default:
+            add(hf, {W_P, W_T});
+            add(f, {W_R, W_XLO});
+            add(d, {W_XHI, W_T64});
+        }
+        return m;
+    }
+    // bytes of the directions that are not allocated yet
+    size_t missing_dirs() const {
+        const int prec = in[0].spec->prec;
+        const size_t n = (size_t)nshift * nsupf;
+        return (prec == SMPQ_FP64 || prec == SMPQ_MIXED ? missing(W_PS, n * sizeof(double2)) : 0) +
+               (prec == SMPQ_FP64 ? 0 : missing(W_PS32, n * sizeof(float2)));
     }
 
     // the slots left in the chunk for iterations of an eb-byte residual

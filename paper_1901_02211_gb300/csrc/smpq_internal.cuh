@@ -71,6 +71,7 @@ struct smpq_ctx {
     std::vector<Tuned> tuned;
     std::string tune_cache; // path of the tuning cache file ("" = none)
     int last_bc = 0;
+    size_t mem_total = 0; // bytes of device memory
     std::vector<cudaEvent_t> prof_ev; // 4 per iteration of one check interval
     double prof_a_ms = 0, prof_b_ms = 0;         // FP32 iterations
     long long prof_a_n = 0, prof_b_n = 0;
