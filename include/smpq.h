@@ -336,6 +336,8 @@ int smpq_trace_dwinv(smpq_ctx *ctx, double *t_re, double *t_im, int on_device, d
  * keyed by a device string (as the library writes it: "<name>/<SMs>sm"), the
  * lattice dims, the batch B and the precision.  One line per entry:
  *   smpq-tune-2|<device>|<nx> <ny> <nz> <nt>|<B>|<precision>|<bc> <tpb_hi> <tpb_lo> <nr> <staged>|<ms>
+ * (smpq-tune-3 for SMPQ_FP64: version-2 lines of that precision belong to other
+ * kernels and are ignored).
  * lookup: SMPQ_OK and shape[5] filled from the last matching well-formed line,
  * SMPQ_ESTATE if the file is missing or has no such line, SMPQ_EINVAL for
  * NULL arguments.  store: appends one line (ms = the tuner's estimate per

@@ -159,8 +159,10 @@ std::string device_key(int dev) {
     return std::string(pr.name) + "/" + std::to_string(pr.multiProcessorCount) + "sm";
 }
 
+// 3: FP64 shapes of the block-fixed-point kernels (their tiles have other sizes, so a
+// number of tiles per block tuned for the FP64 kernels before them means another block)
 std::string cache_key(const char *device, const int dims[4], int B, int precision) {
-    return std::string("smpq-tune-2|") + device + "|" + std::to_string(dims[0]) + " " + std::to_string(dims[1]) +
+    return std::string(precision == SMPQ_FP64 ? "smpq-tune-3|" : "smpq-tune-2|") + device + "|" + std::to_string(dims[0]) + " " + std::to_string(dims[1]) +
            " " + std::to_string(dims[2]) + " " + std::to_string(dims[3]) + "|" + std::to_string(B) + "|" +
            std::to_string(precision) + "|";
 }
