@@ -212,13 +212,14 @@ __global__ void from_half_kernel(const typename HT::h2 *__restrict__ in, const f
     const int j = (int)(i % B), s = (int)(i / B);
     const size_t t = (size_t)(j / BC), jj = (size_t)(j % BC);
     const float n = nin[(t * V + s) * BC + jj];
-    // n * f exactly (24 x 11 bits): the FP32 product and its exact error, in one FP64
-    // addition (conversions and a multiplication there cost 66 cycles a warp each)
+    // n * f exactly (24 x 11 bits): the FP32 product less its exact excess, in one FP64
+    // operation (conversions and a multiplication there cost 66 cycles a warp each);
+    // in this order a product of -0 stays -0
     auto wide = [&](float f) {
         const float p = n * f, a = fabsf(p);
         if (!(a < 3e38f) || (a < 1e-25f && f != 0.f)) // (its error could be subnormal)
             return (double)n * (double)f;
-        return exact_d(p) + exact_d(fmaf(n, f, -p));
+        return exact_d(p) - exact_d(fmaf(-n, f, p));
     };
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
