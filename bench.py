@@ -73,11 +73,12 @@ def _peaks():
 
 def _src_hash(kernel=""):
     """Hash of the files that define a solver kernel (wilson.cuh, df64.cuh,
-    device.cuh, msolve.cuh, and stage.cuh for the staged FP32 kernels `*_st`):
-    traffic figures taken on other sources are void."""
+    device.cuh, msolve.cuh, bfp.cuh for the FP64 kernels `*_bf`, stage.cuh for the
+    staged FP32 kernels `*_st`): traffic figures taken on other sources are void."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1901_02211_gb300", "csrc")
     files = ["df64.cuh", "device.cuh", "msolve.cuh", "wilson.cuh"] + (["stage.cuh"] if "_st[" in kernel else [])
+    files += ["bfp.cuh"] if "_bf[" in kernel else []
     for f in files:
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
@@ -270,12 +271,14 @@ def _kernel_table(prec, stats, V, B, peak_hbm, peak_kind, alu):
     half = prec in (smpq.SMPQ_FP16N, smpq.SMPQ_BF16N)
     lo = {smpq.SMPQ_FP16N: "fp16n", smpq.SMPQ_BF16N: "bf16n"}.get(prec, "fp32")
     st_ = "_st" if stats[-1].get("staged") and lo == "fp32" else ""  # neighbours staged in shared memory
+    bf = prec == smpq.SMPQ_FP64  # block fixed point: 16 bytes a value and 4 a site and source
+    hi = "_bf[fp64]" if bf else "[fp64-accurate]"
     kern = {}
     for key, ms_k, n_k, esz_k, nvec in (
             ("k_apply_a%s[%s]" % (st_, lo), "dslash_ms", "dslash_launches", 8, 2),
             ("k_apply_b%s[%s]" % (st_, lo), "update_ms", "update_launches", 8, b_vecs),
-            ("k_apply_a[fp64-accurate]", "dslash_hi_ms", "dslash_hi_launches", 16, 2),
-            ("k_apply_b[fp64-accurate]", "update_hi_ms", "update_hi_launches", 16, 4)):
+            ("k_apply_a" + hi, "dslash_hi_ms", "dslash_hi_launches", 16, 2),
+            ("k_apply_b" + hi, "update_hi_ms", "update_hi_launches", 16, 4)):
         tot = sum(x[ms_k] for x in stats)
         n = sum(x[n_k] for x in stats)
         if not n or tot <= 0:
@@ -286,7 +289,7 @@ def _kernel_table(prec, stats, V, B, peak_hbm, peak_kind, alu):
             # reconstruct-12 links (96 bytes per site)
             nbytes = V * B * (2 * 52 if key.startswith("k_apply_a") else 2 * 52 + 4 * 96) + V * 96
         else:
-            nbytes = V * B * nvec * 12 * esz_k + V * (link32 if esz_k == 8 else link64)
+            nbytes = V * B * nvec * (12 * esz_k + (4 if bf else 0)) + V * (link32 if esz_k == 8 else link64)
         ms = tot / n
         k = dict(ms=ms, n=n, share_ms=tot / len(stats), bytes=nbytes, bound="hbm", unit="GB/s", peak=peak_hbm,
                  peak_source=peak_kind, achieved=nbytes / (ms / 1000.0) / 1e9)

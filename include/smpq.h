@@ -62,18 +62,25 @@ typedef enum {
 } smpq_status;
 
 typedef enum {
-    SMPQ_FP64 = 0,  /* vectors, dslash and updates in FP64 (reference path) */
+    SMPQ_FP64 = 0,  /* the reference path: vectors and D_W of the solves in 64-bit integers with
+                       one exponent per site and right-hand side (60 bits of the site's
+                       largest component, so that norms and residuals are more accurate
+                       than in FP64 arithmetic; a component that is smaller by 2^k keeps
+                       60 - k bits), scalars, the shifted solutions and y in FP64 */
     SMPQ_FP32 = 1,  /* FP32 vectors and dslash with FP64 reliable updates, FP64 scalars */
     SMPQ_MIXED = 2, /* FP64-accurate iterations (float-float arithmetic on FP64-sized data)
                        until ||r|| <= switch_residual ||b||, then FP32 without residual
-                       replacement; shifted directions in FP64 in the first phase and
-                       FP32 in the second, y in FP64 throughout */
+                       replacement; the residuals are kept on the support (FP64-sized in
+                       the first phase, FP32 in the second) and the shifted solutions
+                       formed from them at the end: y in FP64 in the first phase, the
+                       second phase's share in float-float for a switch_residual up to
+                       2^-8 and in FP64 above */
     SMPQ_FP16N = 3, /* spinor components stored in FP16 and scaled by one FP32 norm per site
                        and right-hand side, links stored as FP16 rows 0 and 1
                        (reconstruct-12), FP32 arithmetic.  smpq_dslash / smpq_time_dslash:
                        the stand-alone D_W in that format.  As a solver precision: the
                        SMPQ_FP32 iterations (FP64 reliable updates, FP32 residual and
-                       shifted directions) with D_W's input p and output t in that
+                       shifted recurrences) with D_W's input p and output t in that
                        format; the shifted systems then keep an error floor near the
                        format's rounding (about 1e-4 relative), far above FP32's. */
     SMPQ_BF16N = 4  /* as SMPQ_FP16N with BF16 storage (floor near 1e-3 relative) */
@@ -97,9 +104,9 @@ typedef struct {
                                4, 8; FP32 columns per thread 1, 2; neighbours staged in shared
                                memory or not, per phase) on the first solve of each batch shape,
                                and use the fastest */
-    int full_support;       /* q(x): keep the shifted directions on every site instead of only where
+    int full_support;       /* q(x): keep the residuals and y on every site instead of only where
                                z = D_W y is read (the ablation of that restriction; same result,
-                               14 full-lattice vectors per source) */
+                               a full-lattice vector per source and iteration) */
     int true_residual;      /* SMPQ_FP64 / SMPQ_MIXED, the base system's true residual
                                |b - (H^2 + s0) x| / |b| (smpq_stats.true_resid):
                                0: not computed (no base solution is kept);

@@ -322,7 +322,7 @@ int compute_classes(smpq_ctx *ctx, const std::vector<int> &classes, double *q_re
     // star support of every class
     int n_sup = 0;
     if ((rc = build_star_support(ctx, ctx->ws[W_SUP], &n_sup))) return rc;
-    // ablation of the star support: shifted directions on every site
+    // ablation of the star support: residuals and y on every site
     const bool full_sup = kind == 0 && ctx->opt.full_support;
     if (full_sup) n_sup = ctx->V;
     const int prec = ctx->opt.precision;

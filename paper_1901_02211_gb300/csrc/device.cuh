@@ -6,6 +6,8 @@
 #include <stdint.h>
 #include "df64.cuh"
 
+constexpr int GB300_SMS = 152;
+
 // ---------------------------------------------------------------- complex helpers
 template <typename T> struct cplx_t;
 template <> struct cplx_t<double> { typedef double2 type; };

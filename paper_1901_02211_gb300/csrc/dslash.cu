@@ -497,7 +497,7 @@ void launch_dslash_fp32_abi(const Geom &g, const void *U, const double *in, void
     const long n = (long)g.V * B;
     abi_to_float_kernel<<<(unsigned)((12 * n + 255) / 256), 256, 0, st>>>((const double2 *)in, (float2 *)field,
                                                                           (size_t)12 * n);
-    const int th = n < 152 * 128 * 4 ? 32 : 128;
+    const int th = n < (long)GB300_SMS * 128 * 4 ? 32 : 128; // at least four blocks an SM, of one warp if need be
     const unsigned nb = (unsigned)((n + th - 1) / th);
     if (dagger)
         dslash_abi_kernel<true><<<nb, th, 0, st>>>(g, (const float2 *)U, (const float2 *)field, (double2 *)out, B,
