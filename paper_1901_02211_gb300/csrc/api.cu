@@ -288,21 +288,19 @@ Shape tune_shape(smpq_ctx *ctx, int B, int prec, int *cached) {
     return s;
 }
 
-// device bytes one right-hand side costs in the solver (full-lattice vectors)
+// device bytes one right-hand side costs in the solver: whole-lattice vectors and, on
+// the support, y and the shifted directions.  The residual history is not among them:
+// batches are sized to 0.6 of the memory, the history has a bound of its own and takes
+// what it finds of the rest (plan_history), so it costs no batch (counted per source it
+// made seven rounds of six for three lattices in one call: 42.4 s instead of 41.0).
 size_t bytes_per_rhs(const smpq_ctx *ctx, int prec, int n_sup, int npoles) {
     const bool half = prec == SMPQ_FP16N || prec == SMPQ_BF16N;
     size_t per = prec == SMPQ_FP32 ? (4 * 8 + 2 * 16)
                  : half            ? (2 * 5 + 2 * 8 + 2 * 16) // p, t: 4 B + a 12th of the 4-byte norm
-                                   : (prec == SMPQ_MIXED ? 4 * 16 + 4 * 8 : 3 * 17); // MIXED: p t r x_hi, p t r x_lo; FP64: p t r, exponents
+                                   : (prec == SMPQ_MIXED ? 4 * 16 + 4 * 8 : 49); // MIXED: p t r x_hi, p t r x_lo; FP64: p t r, exponents
     if (ctx->opt.true_residual && prec == SMPQ_FP64) per += 2 * 16; // x64, t64
-    size_t full = (size_t)ctx->V * 12 * per;
-    // support: y and the residual history, or as much of that as the fields
-    // take (a shorter history needs the shifted directions beside it)
-    const size_t slots = hist_bytes_wanted(prec, ctx->opt.max_iter);
-    const size_t want = (size_t)n_sup * 12 * slots, dirs = (size_t)n_sup * 12 * npoles * 16;
-    // and, per slot, the scalars of every shift
-    const size_t scalars = slots / (prec == SMPQ_FP64 ? 16 : 8) * (npoles * 32 + 24);
-    return full + (size_t)n_sup * 12 * 16 + std::min(want, std::max(full, dirs) + dirs) + scalars;
+    const size_t eb = (prec == SMPQ_FP32 || half) ? 8 : (prec == SMPQ_MIXED ? 16 + 8 : 16); // MIXED: FP64 and FP32 directions
+    return (size_t)ctx->V * 12 * per + (size_t)n_sup * 12 * (npoles * eb + 16);
 }
 
 // kind 0: q^SMP(x) of Eq. 16; kind 1: SMP estimate of diag D_W^{-1}

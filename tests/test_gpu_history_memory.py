@@ -84,3 +84,32 @@ def test_fields_come_before_the_history(torch):
     got = run(112 * values)
     # chunks sum the same history in other portions
     assert np.abs(got - want).max() <= 1e-11 * np.abs(want).max()
+
+
+def test_history_costs_no_batch(torch):
+    """192 mixed sources of r = 2 on 8^3x16 cost 28.9 MB each (96 bytes a value on the
+    lattice, 352 on 9/16 of it): 10.3 GB free, of which batches take 0.6, hold them in
+    one batch, whatever the history would like."""
+    from paper_1901_02211_gb300 import Session, smpq
+    from synth import make_config
+    cfg = make_config("flux8x16")
+    with open(os.path.join(os.path.dirname(__file__), "golden", "spectra.json")) as f:
+        spec = json.load(f)["flux8x16"]
+    got = []
+    for target in (0, 10300 << 20):
+        with Session(device=0, stream=torch.cuda.current_stream().cuda_stream, precision=smpq.SMPQ_MIXED,
+                     autotune=0) as s:
+            s.load_gauge(cfg["dims"], cfg["U"])
+            s.set_spectrum(0.98 * spec["lmin2"], 1.02 * spec["lmax2"])
+            s.build_sources(2, 0)
+            block = None
+            if target:
+                block = torch.empty(_free(torch)[0] - target, dtype=torch.uint8, device="cuda")
+            try:
+                q, Q, st = s.compute_qx()
+            finally:
+                del block
+                torch.cuda.empty_cache()
+        assert st["n_batches"] == 1
+        got.append(q)
+    assert np.abs(got[1] - got[0]).max() <= 1e-11 * np.abs(got[0]).max()
