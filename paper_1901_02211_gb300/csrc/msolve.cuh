@@ -1538,8 +1538,10 @@ __global__ void __launch_bounds__(256) k_hist_y(HistLat L, const double *__restr
 // block at once, and serve the HROWS values of a thread from there (read from
 // global memory shift by shift they were the latency of the whole kernel: 100
 // ms of a 266 ms solve of three r = 2 lattices).
-constexpr int HROWS = 2, NG = 14;
-template <int BC, typename V> struct HistTile {
+//   NG is 14, or 1 for solves of one shift (the trace: with 14 it took 140 ms for 192
+// mixed sources of 8^3x16, 124 with 1).
+constexpr int HROWS = 2;
+template <int BC, typename V, int NG> struct HistTile {
     typedef TileMap<BC> TM;
     int jj, j, cls;      // column within the tile and the solve, its class
     size_t e[HROWS];     // elements, valid where ok
@@ -1578,14 +1580,14 @@ template <int BC> static dim3 hist_grid(const HistLat &L) {
 // FP64 ones of 66), rounded to FP32 at the end.  The weights then fall like
 // (|r_n| / |r_k|)^2: one below the FP32 range belongs to a term that far below
 // the last ones.
-template <typename C, int BC, bool F32>
+template <typename C, int BC, bool F32, int NG>
 __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_p(HistLat L, const double *__restrict__ hp,
                                                                  const double *__restrict__ d0,
                                                                  double2 *__restrict__ ps,
                                                                  float2 *__restrict__ ps32) {
     constexpr int HK = 8;
     __shared__ double sm[HK][NG][BC];
-    const HistTile<BC, double> T(L);
+    const HistTile<BC, double, NG> T(L);
     for (int i0 = 0; i0 < L.nshift; i0 += NG) {
         for (int q = 0; q < HROWS; ++q) {
             double2 acc[F32 ? 1 : NG];
@@ -1609,7 +1611,7 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_p(HistLat L, cons
             }
             for (int k0 = 0; k0 < L.n; k0 += HK) {
                 __syncthreads();
-                HistTile<BC, double>::template load<HK>(L, hp, k0, i0, sm, 0.0);
+                HistTile<BC, double, NG>::template load<HK>(L, hp, k0, i0, sm, 0.0);
                 __syncthreads();
                 if (!T.ok[q]) continue;
 #pragma unroll
@@ -1674,15 +1676,15 @@ __global__ void k_hist_coef(int n, int nshift, int B, int j0, int Bl, const Shif
 // y starts here (SMPQ_FP32 and the half storage), the sums are FP64.
 constexpr double HIST_FF_THETA = 1.0 / 256;
 inline bool hist_exact(int prec, double theta) { return prec != SMPQ_MIXED || theta > HIST_FF_THETA; }
-template <int BC, bool EXACT>
+template <int BC, bool EXACT, int NG>
 __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_run(HistLat L, const double *__restrict__ ca,
                                                                    const float4 *__restrict__ ct,
                                                                    float2 *__restrict__ ps32,
                                                                    double2 *__restrict__ y, bool last) {
-    constexpr int HK = EXACT ? 2 : 4;
+    constexpr int HK = NG == 1 ? 8 : EXACT ? 2 : 4;
     __shared__ float4 sm[HK][NG][BC];
     __shared__ double sa[EXACT ? HK : 1][NG][BC];
-    const HistTile<BC, float4> T(L);
+    const HistTile<BC, float4, NG> T(L);
     for (int i0 = 0; i0 < L.nshift; i0 += NG) {
         float2 p[HROWS][NG], s[HROWS], d[HROWS];
         double2 yv[HROWS];
@@ -1702,8 +1704,8 @@ __global__ void __launch_bounds__(TileMap<BC>::THREADS) k_hist_run(HistLat L, co
         }
         for (int k0 = 0; k0 < L.n; k0 += HK) {
             __syncthreads();
-            HistTile<BC, float4>::template load<HK>(L, ct, k0, i0, sm, make_float4(0.f, 0.f, 0.f, 0.f));
-            if constexpr (EXACT) HistTile<BC, double>::template load<HK>(L, ca, k0, i0, sa, 0.0);
+            HistTile<BC, float4, NG>::template load<HK>(L, ct, k0, i0, sm, make_float4(0.f, 0.f, 0.f, 0.f));
+            if constexpr (EXACT) HistTile<BC, double, NG>::template load<HK>(L, ca, k0, i0, sa, 0.0);
             __syncthreads();
             float2 rv[HK][HROWS];
 #pragma unroll
@@ -2361,6 +2363,10 @@ template <int BC> struct Solve {
         L.first = hfirst;
         return L;
     }
+    template <typename F> void shift_groups(F launch) const {
+        if (nshift == 1) launch(std::integral_constant<int, 1>());
+        else launch(std::integral_constant<int, 14>());
+    }
     int hist_next(bool last, int launched) {
         ctx->launches += launched;
         if (!last) cudaMemsetAsync(sc.slot, 0, (size_t)B * sizeof(int), st);
@@ -2387,9 +2393,14 @@ template <int BC> struct Solve {
             float2 *ps32 = (float2 *)ws[W_PS32].p + s0[l];
             const unsigned nb = (unsigned)((L.ne + 255) / 256);
             k_hist_y<C, BC><<<nb, 256, 0, st>>>(L, hw, hv0, ps, y + s0[l]);
-            if (next == 1) k_hist_p<C, BC, false><<<hist_grid<BC>(L), TileMap<BC>::THREADS, 0, st>>>(L, sc.ho, hd0, ps, ps32);
-            if constexpr (std::is_same<C, df64c>::value)
-                if (next == 2) k_hist_p<C, BC, true><<<hist_grid<BC>(L), TileMap<BC>::THREADS, 0, st>>>(L, sc.ho, hd0, ps, ps32);
+            const dim3 grid = hist_grid<BC>(L);
+            const int TH = TileMap<BC>::THREADS;
+            shift_groups([&](auto ng) {
+                constexpr int NG = decltype(ng)::value;
+                if (next == 1) k_hist_p<C, BC, false, NG><<<grid, TH, 0, st>>>(L, sc.ho, hd0, ps, ps32);
+                if constexpr (std::is_same<C, df64c>::value)
+                    if (next == 2) k_hist_p<C, BC, true, NG><<<grid, TH, 0, st>>>(L, sc.ho, hd0, ps, ps32);
+            });
         }
         return hist_next(next == 0, 1 + (next ? 3 : 2) * nl);
     }
@@ -2407,8 +2418,11 @@ template <int BC> struct Solve {
             float2 *ps32 = (float2 *)ws[W_PS32].p + s0[l];
             const dim3 nb = hist_grid<BC>(L);
             const int TH = TileMap<BC>::THREADS;
-            if (exact) k_hist_run<BC, true><<<nb, TH, 0, st>>>(L, sc.ho, hct, ps32, y + s0[l], last);
-            else k_hist_run<BC, false><<<nb, TH, 0, st>>>(L, sc.ho, hct, ps32, y + s0[l], last);
+            shift_groups([&](auto ng) {
+                constexpr int NG = decltype(ng)::value;
+                if (exact) k_hist_run<BC, true, NG><<<nb, TH, 0, st>>>(L, sc.ho, hct, ps32, y + s0[l], last);
+                else k_hist_run<BC, false, NG><<<nb, TH, 0, st>>>(L, sc.ho, hct, ps32, y + s0[l], last);
+            });
         }
         return hist_next(last, 2 * nl);
     }

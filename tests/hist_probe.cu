@@ -57,14 +57,18 @@ extern "C" int hist_probe(int fp32, double theta, int n, int nshift, int n_sup, 
     if (fp32) {
         L.h = dr32.p;
         k_hist_coef<<<(unsigned)((rows + 255) / 256), 256>>>(n, nshift, B, 0, B, dsp.p, sc, ct.p);
-        if (hist_exact(SMPQ_MIXED, theta)) k_hist_run<B, true><<<grid, TH>>>(L, ho.p, ct.p, dp32.p, dy.p, true);
-        else k_hist_run<B, false><<<grid, TH>>>(L, ho.p, ct.p, dp32.p, dy.p, true);
+        const bool exact = hist_exact(SMPQ_MIXED, theta);
+        if (nshift == 1 && exact) k_hist_run<B, true, 1><<<grid, TH>>>(L, ho.p, ct.p, dp32.p, dy.p, true);
+        else if (nshift == 1) k_hist_run<B, false, 1><<<grid, TH>>>(L, ho.p, ct.p, dp32.p, dy.p, true);
+        else if (exact) k_hist_run<B, true, 14><<<grid, TH>>>(L, ho.p, ct.p, dp32.p, dy.p, true);
+        else k_hist_run<B, false, 14><<<grid, TH>>>(L, ho.p, ct.p, dp32.p, dy.p, true);
     } else {
         L.h = dr.p;
         k_hist_w<<<(nshift * B + 127) / 128, 128>>>(n, nshift, B, 0, B, dsp.p, sc, v0.p, d0.p, false);
         k_hist_sum<<<(unsigned)(((size_t)(n + 1) * B + 255) / 256), 256>>>(n, nshift, B, hz.p, v0.p, hw.p);
         k_hist_y<double2, B><<<(unsigned)((ne + 255) / 256), 256>>>(L, hw.p, v0.p, dps.p, dy.p);
-        k_hist_p<double2, B, false><<<grid, TH>>>(L, ho.p, d0.p, dps.p, dp32.p);
+        if (nshift == 1) k_hist_p<double2, B, false, 1><<<grid, TH>>>(L, ho.p, d0.p, dps.p, dp32.p);
+        else k_hist_p<double2, B, false, 14><<<grid, TH>>>(L, ho.p, d0.p, dps.p, dp32.p);
         dps.get(ps);
     }
     dy.get(y);

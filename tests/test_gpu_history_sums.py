@@ -70,7 +70,7 @@ def test_directions_after_one_iteration(probe, nshift, scale):
         assert (err <= 2 * U * (np.abs(b * p) + np.abs(z * q))).all()
 
 
-@pytest.mark.parametrize("n,nshift", [(3, 2), (19, 14), (40, 17)])
+@pytest.mark.parametrize("n,nshift", [(3, 2), (19, 14), (40, 17), (37, 1)])
 def test_chunk_of_fp64_iterations(probe, n, nshift):
     """y and the directions against the recurrences in extended precision.  A weight has
     up to 5 roundings per iteration (zeta ratio twice, beta, alpha, the product) and one
@@ -80,7 +80,8 @@ def test_chunk_of_fp64_iterations(probe, n, nshift):
     r, ps, y = _fields(rng, n, nshift, ne)
     zn, zo = rng.uniform(0.5, 1, (2, n, nshift, 12))
     alpha, beta = rng.uniform(0.5, 1, (2, n, 12))
-    zn[n // 2:, nshift - 1] = 0  # the last shift has converged
+    if nshift > 1:
+        zn[n // 2:, nshift - 1] = 0  # the last shift has converged
     c = rng.uniform(0.1, 1, nshift)
     gy, gp = probe(False, 0, c, zn, zo, alpha, beta, r, ps, y)
     col = _columns(ne)
@@ -125,12 +126,12 @@ def test_share_of_fp32_iterations(probe, theta, nshift):
         assert (err <= (3 + nshift) * U * np.abs(terms).sum(0)).all()
 
 
-@pytest.mark.parametrize("n", [1, 7, 30])
-def test_share_below_a_small_switch_residual(probe, n):
+@pytest.mark.parametrize("n,nshift", [(1, 14), (7, 14), (30, 14), (30, 1)])
+def test_share_below_a_small_switch_residual(probe, n, nshift):
     """At the largest switch residual with float-float sums, y of that many times the
     share: within the FP64 sums' own bound (an addition per shift and iteration)."""
     rng = np.random.default_rng(n)
-    ne, nshift = 144 * 3, 14
+    ne = 144 * 3
     r, ps, _ = _fields(rng, n, nshift, ne)
     r, ps = (x.astype(np.complex64).astype(complex) for x in (r, ps))
     zeta = np.broadcast_to(rng.uniform(0.5, 1, (1, nshift, 12)), (n, nshift, 12)).copy()
