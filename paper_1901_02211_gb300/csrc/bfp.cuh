@@ -325,6 +325,8 @@ __device__ __forceinline__ void bf_hop(bool back, const int4 *__restrict__ U, co
 }
 
 // acc * 2^(eref + 4) = hop(s); eref = the largest exponent of s and its neighbours
+// (neighbours and exponents stay in registers here; BfStar below forms them again,
+// which in these kernels spills more: 278 against 271 ms for the trace of 8^3x16)
 template <bool DAG, typename Off>
 __device__ __forceinline__ void bf_wilson(const Geom &g, const int4 *__restrict__ U, const bfc *__restrict__ in,
                                           const int *__restrict__ ein, const Off &off, int s, int one, bfc acc[12],
