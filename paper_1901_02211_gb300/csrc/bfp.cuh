@@ -324,42 +324,49 @@ __device__ __forceinline__ void bf_hop(bool back, const int4 *__restrict__ U, co
     }
 }
 
+// where a site lies at the lattice's edges, and its neighbours
+struct BfSite {
+    unsigned edges; // bit 2 mu: last coordinate, bit 2 mu + 1: first one
+    __device__ __forceinline__ BfSite(const Geom &g, int s) {
+        const SiteCoords xc(g, s);
+        edges = 0;
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu)
+            edges |= (xc.x[mu] == g.n[mu] - 1 ? 1u : 0u) << (2 * mu) | (xc.x[mu] == 0 ? 2u : 0u) << (2 * mu);
+    }
+    // k = 2 mu: forward in direction mu, 2 mu + 1: backward
+    __device__ __forceinline__ bool edge(int k) const { return edges >> k & 1; }
+    __device__ __forceinline__ int neighbour(const Geom &g, int s, int k) const {
+        const int st = g.stride[k >> 1], far = (g.n[k >> 1] - 1) * st;
+        return k & 1 ? (edge(k) ? s + far : s - st) : (edge(k) ? s - far : s + st);
+    }
+};
+
 // acc * 2^(eref + 4) = hop(s); eref = the largest exponent of s and its neighbours
-// (neighbours and exponents stay in registers here; BfStar below forms them again,
-// which in these kernels spills more: 278 against 271 ms for the trace of 8^3x16)
 template <bool DAG, typename Off>
 __device__ __forceinline__ void bf_wilson(const Geom &g, const int4 *__restrict__ U, const bfc *__restrict__ in,
                                           const int *__restrict__ ein, const Off &off, int s, int one, bfc acc[12],
                                           int &eown, int &eref) {
-    const SiteCoords xc(g, s);
-    int nbk[8];
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        const int n = g.n[mu], st = g.stride[mu], c = xc.x[mu];
-        nbk[2 * mu] = c == n - 1 ? s - (n - 1) * st : s + st;
-        nbk[2 * mu + 1] = c == 0 ? s + (n - 1) * st : s - st;
-    }
-    int en[8];
+    const BfSite x(g, s);
+    int nb[8], en[8];
     eown = eref = ein[off.exp(s)];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        en[k] = ein[off.exp(nbk[k])];
+        nb[k] = x.neighbour(g, s, k);
+        en[k] = ein[off.exp(nb[k])];
         eref = max(eref, en[k]);
     }
 #pragma unroll
     for (int c = 0; c < 12; ++c) acc[c] = {0, 0};
     auto dir = [&](auto mc) {
         constexpr int MU = decltype(mc)::value;
-        const int n = g.n[MU], c = xc.x[MU];
         const bool anti = g.bcf[MU] < 0;
         // forward: (1 - g) [DAG: (1 + g)], backward: (1 + g) [DAG: (1 - g)]
 #pragma unroll 1
         for (int bk = 0; bk < 2; ++bk) {
-            const bool back = bk != 0;
-            const int nb = back ? nbk[2 * MU + 1] : nbk[2 * MU];
-            const int en1 = back ? en[2 * MU + 1] : en[2 * MU];
-            bf_hop<MU, DAG>(back, U, in, off, g.V, nb, back ? nb : s, min(eref - en1, 63),
-                               anti && c == (back ? 0 : n - 1), one, acc);
+            const int n = bk ? nb[2 * MU + 1] : nb[2 * MU], e = bk ? en[2 * MU + 1] : en[2 * MU];
+            bf_hop<MU, DAG>(bk != 0, U, in, off, g.V, n, bk ? n : s, min(eref - e, 63), anti && x.edge(2 * MU + bk), one,
+                            acc);
         }
     };
     dir(std::integral_constant<int, 0>());
@@ -371,22 +378,16 @@ __device__ __forceinline__ void bf_wilson(const Geom &g, const int4 *__restrict_
 // The stand-alone D_W's exponents carry in their lowest bit whether the nonzero
 // components of the site span 2^12 and more.
 __device__ __forceinline__ int bf_tag(int e, bool wide) { return 2 * e + wide; }
-// What it knows of a site before it reads any component: where it lies at the
-// lattice's edges, its exponent and the star's largest, whether every neighbour is
-// zero (D_W then changes nothing).  Neighbours and their exponents are formed again
-// in each hop: kept over the eight hops they were 160 bytes of spills.
-struct BfStar {
-    unsigned edges; // bit 2 mu: last coordinate, bit 2 mu + 1: first one
+// What it knows of a site before it reads any component: its exponent and the star's
+// largest, whether every neighbour is zero (D_W then changes nothing).  Neighbours and
+// their exponents are formed again in each hop: kept over the eight hops they were 160
+// bytes of spills.
+struct BfStar : BfSite {
     int eown, eref;
     bool alone;
     bool uneven; // bf_dw_fine is likely to find a small component: tagged, or only one or two large neighbours
     template <typename Off>
-    __device__ __forceinline__ BfStar(const Geom &g, const int *__restrict__ tag, const Off &off, int s) {
-        const SiteCoords xc(g, s);
-        edges = 0;
-#pragma unroll
-        for (int mu = 0; mu < 4; ++mu)
-            edges |= (xc.x[mu] == g.n[mu] - 1 ? 1u : 0u) << (2 * mu) | (xc.x[mu] == 0 ? 2u : 0u) << (2 * mu);
+    __device__ __forceinline__ BfStar(const Geom &g, const int *__restrict__ tag, const Off &off, int s) : BfSite(g, s) {
         int en[8], top = BF_ZERO, large = 0;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -401,12 +402,6 @@ struct BfStar {
         alone = top <= BF_ZERO / 2;
         uneven = !alone && ((own & 1) || large <= 2);
     }
-    // k = 2 mu: forward in direction mu, 2 mu + 1: backward
-    __device__ __forceinline__ int neighbour(const Geom &g, int s, int k) const {
-        const int st = g.stride[k >> 1], far = (g.n[k >> 1] - 1) * st;
-        const bool edge = edges >> k & 1;
-        return k & 1 ? (edge ? s + far : s - st) : (edge ? s - far : s + st);
-    }
     // a block in the star is marked bad
     __device__ __forceinline__ bool bad() const { return eref >= BF_BAD / 2; }
 };
@@ -420,7 +415,7 @@ __device__ __forceinline__ void bf_dir(const BfStar &x, const Geom &g, const int
     for (int bk = 0; bk < 2; ++bk) {
         const int k = 2 * MU + bk, nb = x.neighbour(g, s, k);
         bf_hop<MU, DAG, true>(bk != 0, U, in, off, g.V, nb, bk ? nb : s, min(x.eref - (tag[off.exp(nb)] >> 1), 63),
-                              anti && (x.edges >> k & 1), one, acc, size);
+                              anti && x.edge(k), one, acc, size);
     }
 }
 // The eight hops of the star x and their sizes, or (split) by four groups of GT
