@@ -247,7 +247,7 @@ __device__ __forceinline__ unsigned bf_swap(unsigned z) { return (z >> 16) | (z 
 // 210 against 178 ms for six classes of 8^3x16, "no instruction" the first stall).
 // links: int4 {re high, re low, im high, im low} per element
 // SIZES: size[c] += the leading bits of |re| (low half) and |im| (high half) of
-// component c's term, in units of 2^48 (bf_small)
+// component c's term, in units of 2^48 (bf_dw_fine)
 template <int MU, bool DAG, bool SIZES = false, typename Off>
 __device__ __forceinline__ void bf_hop(bool back, const int4 *__restrict__ U, const bfc *__restrict__ in,
                                           const Off &off, int Vl, int nb, int ls, int n, bool flip, int one,

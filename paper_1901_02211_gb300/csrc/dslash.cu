@@ -353,10 +353,10 @@ static __device__ __noinline__ void dw_site_fp64_warp(const Geom &g, const doubl
 constexpr int FP64_WARP_MAX = 8;
 
 // One thread per site and column; bound by the integer pipe (8^3x16: 51 us for 12
-// columns, 3.94 ms for 1000; with 128 registers and four blocks an SM 57 us and
-// 4.02 ms, the sizes of the terms spill).  Sites whose star
-// holds a bad block, and those where bf_dw_fine finds a component too small for
-// the common unit, are done in FP64 (`in` is read there: it may not overlap out).
+// columns, 3.9 ms for 1000; with 128 registers and four blocks an SM 57 us and 4.0 ms,
+// the sizes of the terms spill).  Sites whose star holds a bad block, and those where
+// bf_dw_fine finds a component too small for the common unit, are done in FP64 (`in`
+// is read there: it may not overlap out).
 // A warp whose sites look uneven for the most part does not try (fields of sites or
 // components of very different size: 243 to 250 us a call on 12 columns of 8^3x16
 // with links that do not mix them, 265 to 271 with both).

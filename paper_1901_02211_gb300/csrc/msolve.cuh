@@ -2293,7 +2293,9 @@ template <int BC> struct Solve {
                 if ((eb == sizeof(double2) && (rc = hist_dirs(W_PS, sizeof(double2)))) ||
                     (!fp64 && (rc = hist_dirs(W_PS32, sizeof(float2)))))
                     return rc;
-                want = std::min(want, std::max(eb, room() / 4 * 3 / nsupf / eb * eb));
+                // (a history kept from the same call before stays as it is: the same chunks)
+                const size_t give = std::max(room() / 4 * 3, hist.bytes);
+                want = std::min(want, std::max(eb, give / nsupf / eb * eb));
             }
             if (hist.bytes < want * nsupf && (rc = ensure(ctx, hist, want * nsupf))) return rc;
         }

@@ -74,6 +74,7 @@ def test_fields_come_before_the_history(torch):
                 block = torch.empty(free - target, dtype=torch.uint8, device="cuda")
             try:
                 q, Q, st = s.compute_qx(classes=classes)
+                assert np.array_equal(q, s.compute_qx(classes=classes)[0])  # the same chunks again
             finally:
                 del block
                 torch.cuda.empty_cache()
